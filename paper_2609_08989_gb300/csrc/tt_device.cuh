@@ -10,6 +10,7 @@
 #include <cuda_runtime.h>
 
 #include "tt_internal.h"
+#include "tt_soft64.cuh"
 
 namespace tt {
 
@@ -100,23 +101,33 @@ struct State {
 // (the same expressions regrouped: 4 fewer FP64 operations per evaluation).
 // One reciprocal serves 1/Sigma, 1/Delta and 1/sin^2.
 // ---------------------------------------------------------------------------
-// The flow given s = sin(theta), c = cos(theta) of the state.
+// The flow given s = sin(theta), c = cos(theta) of the state, with the products
+// formed by m (tt_soft64.cuh).  For IntMul the checks leave every product that
+// is not checked itself with two factors that are normal: r, p_r, s, c and SD
+// lie in 2^+-100, so Sigma, Delta, 1/Sigma, 1/Delta and 1/sin^2 lie in 2^+-300.
+// K cancels to ~1e-16 of its terms, at times to zero: its product with 1/Sigma
+// is always a plain one.
+template <class Mul>
 __device__ __forceinline__ void kerr_flow64_sc(const KerrK& k, const RayConst& R, const State& y, double s,
-                                               double c, State& f, double& H) {
+                                               double c, State& f, double& H, Mul& m) {
     const double r = y.r;
-    const double s2 = s * s, c2 = c * c, sc = s * c;
-    const double r2 = r * r;
+    m.see(r);
+    m.see(y.pr);
+    m.see(s);
+    m.see(c);
+    const double s2 = m.mul(s, s), c2 = m.mul(c, c), sc = m.mul(s, c);
+    const double r2 = m.mul(r, r);
     const double Sig = fma(k.a2, c2, r2);
     const double Del = fma(r, r - k.twoM, k.a2);
     const double A = fma(fma(r, r, k.a2), R.pt, R.apph);
-    const double SD = Sig * Del;
-    const double inv = rcp64(SD * s2);
-    const double w = inv * s2;                       // 1 / (Sigma Delta)
-    const double iS = w * Del;                       // 1 / Sigma
-    const double iD = w * Sig;                       // 1 / Delta
-    const double u = inv * SD;                       // 1 / sin^2
-    const double pr2 = y.pr * y.pr;
-    const double AiD = A * iD;
+    const double SD = m.chk(Sig, Del);
+    const double inv = rcp64(m.mul(SD, s2));
+    const double w = m.mul(inv, s2);                 // 1 / (Sigma Delta)
+    const double iS = m.mul(w, Del);                 // 1 / Sigma
+    const double iD = m.mul(w, Sig);                 // 1 / Delta
+    const double u = m.mul(inv, SD);                 // 1 / sin^2
+    const double pr2 = m.mul(y.pr, y.pr);
+    const double AiD = m.chk(A, iD);
     double K = fma(R.a2pt2, s2, R.c0);
     K = fma(R.pph2, u, K);
     K = fma(y.pth, y.pth, K);
@@ -126,19 +137,20 @@ __device__ __forceinline__ void kerr_flow64_sc(const KerrK& k, const RayConst& R
     H = 0.5 * H2;
     const double q1 = fma(R.pt2, AiD, H2);
     const double q2 = fma(AiD, AiD, pr2);
-    const double t1 = fma(-R.pph2, u * u, R.a2pt2);
+    const double t1 = fma(-R.pph2, m.mul(u, u), R.a2pt2);
     const double t2 = fma(k.a2, H2, t1);
-    f.r = (Del * y.pr) * iS;
-    f.th = y.pth * iS;
-    f.pr = fma(r, q1, -((r - k.M) * q2)) * iS;
-    f.pth = -(sc * iS) * t2;
+    f.r = m.mul(m.mul(Del, y.pr), iS);
+    f.th = m.chk(y.pth, iS);
+    f.pr = m.chk(fma(r, q1, -m.chk(r - k.M, q2)), iS);
+    f.pth = m.chk(-m.mul(sc, iS), t2);
 }
 
 __device__ __forceinline__ void kerr_flow64(const KerrK& k, const RayConst& R, const State& y, State& f,
                                             double& H) {
     double s, c;
     sincos(y.th, &s, &c);
-    kerr_flow64_sc(k, R, y, s, c, f, H);
+    FpMul m;
+    kerr_flow64_sc(k, R, y, s, c, f, H, m);
 }
 
 // sin and cos of theta from those of a nearby theta0 (the start of the step):
@@ -147,21 +159,24 @@ __device__ __forceinline__ void kerr_flow64(const KerrK& k, const RayConst& R, c
 // against ~28 for a full sincos (measured on GB300); through d^5 and d^6 for
 // |d| < 0.01 (truncation below 2e-18, three fused multiply-adds fewer); farther
 // away, sincos.  (The tier thresholds are compared on the integer pipe.)
-__device__ __forceinline__ void sincos_near(double th, double th0, double s0, double c0, double& s, double& c) {
+// (theta = theta0, d = 0, fails IntMul's check of sin d.)
+template <class Mul>
+__device__ __forceinline__ void sincos_near(double th, double th0, double s0, double c0, double& s, double& c,
+                                            Mul& m) {
     const double d = th - th0;
     if (abs_below_hi(d, kHi0p01)) {
-        const double d2 = d * d;
-        const double sd = d * fma(d2, fma(d2, 1.0 / 120.0, -1.0 / 6.0), 1.0);
+        const double d2 = m.mul(d, d);
+        const double sd = m.chk(d, fma(d2, fma(d2, 1.0 / 120.0, -1.0 / 6.0), 1.0));
         const double cd = fma(d2, fma(d2, fma(d2, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
-        s = fma(s0, cd, c0 * sd);
-        c = fma(c0, cd, -(s0 * sd));
+        s = fma(s0, cd, m.mul(c0, sd));
+        c = fma(c0, cd, -m.mul(s0, sd));
     } else if (abs_below_hi(d, kHi0p1)) {
-        const double d2 = d * d;
-        const double sd =
-            d * fma(d2, fma(d2, fma(d2, fma(d2, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0), -1.0 / 6.0), 1.0);
+        const double d2 = m.mul(d, d);
+        const double sd = m.chk(
+            d, fma(d2, fma(d2, fma(d2, fma(d2, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0), -1.0 / 6.0), 1.0));
         const double cd = fma(d2, fma(d2, fma(d2, fma(d2, 1.0 / 40320.0, -1.0 / 720.0), 1.0 / 24.0), -0.5), 1.0);
-        s = fma(s0, cd, c0 * sd);
-        c = fma(c0, cd, -(s0 * sd));
+        s = fma(s0, cd, m.mul(c0, sd));
+        c = fma(c0, cd, -m.mul(s0, sd));
     } else {
         sincos(th, &s, &c);
     }

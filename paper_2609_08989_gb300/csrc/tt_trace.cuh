@@ -59,32 +59,43 @@ __device__ __forceinline__ double step_factor(double err2) {
 // On the closed-form metric (METRIC 0) the stages take sin and cos of theta
 // from (s0, c0) of the step start by angle addition, and the new point's are
 // returned in (sn, cn) for the next step (first same as last).
-template <int METRIC>
+template <int METRIC, class Mul>
 __device__ __forceinline__ void flow64_near(const ImageDesc& d, const KerrK& kk, const RayConst& R, const State& y,
                                             double th0, double s0, double c0, State& f, double& H, double& s,
-                                            double& c) {
+                                            double& c, Mul& m) {
     if constexpr (METRIC == 0) {
-        sincos_near(y.th, th0, s0, c0, s, c);
-        kerr_flow64_sc(kk, R, y, s, c, f, H);
+        sincos_near(y.th, th0, s0, c0, s, c, m);
+        kerr_flow64_sc(kk, R, y, s, c, f, H, m);
     } else {
         flow64<METRIC>(d, kk, R, y, f, H);
     }
 }
 
-template <int METRIC, int METHOD = 0>
+// Products with the flow k1, the coefficients h a_ij and (s0, c0) are formed by
+// m: for IntMul, k1, h, s0 and c0 are checked here, k2 .. k6 in their flows.
+template <int METRIC, int METHOD, class Mul>
 __device__ __forceinline__ void rk_step64(const ImageDesc& d, const KerrK& kk, const RayConst& R,
                                            const State& y, const State& k1, double h, State& yn,
-                                           State& kn, double& Hn, State& err, double s0 = 0.0, double c0 = 1.0,
-                                           double* sn = nullptr, double* cn = nullptr) {
+                                           State& kn, double& Hn, State& err, double s0, double c0,
+                                           double& sn, double& cn, Mul& m) {
     using T = RK<METHOD>;
     State k2, k3, k4, k5, k6, ys;
     double Hs, ss = s0, cs = c0;
+    m.see(h);
+    m.see(k1.r);
+    m.see(k1.th);
+    m.see(k1.pr);
+    m.see(k1.pth);
+    if (METRIC == 0) {
+        m.see(s0);
+        m.see(c0);
+    }
 #define TT_STAGE(dst, expr_r, expr_t, expr_p, expr_q)                                \
     ys.r = fma(h, (expr_r), y.r);                                                    \
     ys.th = fma(h, (expr_t), y.th);                                                  \
     ys.pr = fma(h, (expr_p), y.pr);                                                  \
     ys.pth = fma(h, (expr_q), y.pth);                                                \
-    flow64_near<METRIC>(d, kk, R, ys, y.th, s0, c0, dst, Hs, ss, cs);
+    flow64_near<METRIC>(d, kk, R, ys, y.th, s0, c0, dst, Hs, ss, cs, m);
 // stages 2-4: coefficients pre-multiplied by h (one multiply each, shared by
 // the four components), the stage point an FMA chain from y
 #define TT_PSTAGE(dst, EXPR)                                                         \
@@ -92,15 +103,15 @@ __device__ __forceinline__ void rk_step64(const ImageDesc& d, const KerrK& kk, c
     ys.th = EXPR(th);                                                                \
     ys.pr = EXPR(pr);                                                                \
     ys.pth = EXPR(pth);                                                              \
-    flow64_near<METRIC>(d, kk, R, ys, y.th, s0, c0, dst, Hs, ss, cs);
-    const double h21 = h * T::a21, h31 = h * T::a31, h32 = h * T::a32;
-    const double h41 = h * T::a41, h42 = h * T::a42, h43 = h * T::a43;
+    flow64_near<METRIC>(d, kk, R, ys, y.th, s0, c0, dst, Hs, ss, cs, m);
+    const double h21 = m.mul(h, T::a21), h31 = m.mul(h, T::a31), h32 = m.mul(h, T::a32);
+    const double h41 = m.mul(h, T::a41), h42 = m.mul(h, T::a42), h43 = m.mul(h, T::a43);
 #define TT_P2(f) fma(h21, k1.f, y.f)
 #define TT_P3(f) fma(h32, k2.f, fma(h31, k1.f, y.f))
 #define TT_P4(f) fma(h43, k3.f, fma(h42, k2.f, fma(h41, k1.f, y.f)))
-#define TT_C5(f) fma(T::a54, k4.f, fma(T::a53, k3.f, fma(T::a52, k2.f, T::a51 * k1.f)))
-#define TT_C6(f) fma(T::a65, k5.f, fma(T::a64, k4.f, fma(T::a63, k3.f, fma(T::a62, k2.f, T::a61 * k1.f))))
-#define TT_C7(f) fma(T::b6, k6.f, TT_MAC(T::b5, k5.f, fma(T::b4, k4.f, fma(T::b3, k3.f, T::b1 * k1.f))))
+#define TT_C5(f) fma(T::a54, k4.f, fma(T::a53, k3.f, fma(T::a52, k2.f, m.mul(k1.f, T::a51))))
+#define TT_C6(f) fma(T::a65, k5.f, fma(T::a64, k4.f, fma(T::a63, k3.f, fma(T::a62, k2.f, m.mul(k1.f, T::a61)))))
+#define TT_C7(f) fma(T::b6, k6.f, TT_MAC(T::b5, k5.f, fma(T::b4, k4.f, fma(T::b3, k3.f, m.mul(k1.f, T::b1)))))
     TT_PSTAGE(k2, TT_P2)
     TT_PSTAGE(k3, TT_P3)
     TT_PSTAGE(k4, TT_P4)
@@ -110,14 +121,12 @@ __device__ __forceinline__ void rk_step64(const ImageDesc& d, const KerrK& kk, c
     yn.th = fma(h, TT_C7(th), y.th);
     yn.pr = fma(h, TT_C7(pr), y.pr);
     yn.pth = fma(h, TT_C7(pth), y.pth);
-    flow64_near<METRIC>(d, kk, R, yn, y.th, s0, c0, kn, Hn, ss, cs);
-    if (sn) {
-        *sn = ss;
-        *cn = cs;
-    }
+    flow64_near<METRIC>(d, kk, R, yn, y.th, s0, c0, kn, Hn, ss, cs, m);
+    sn = ss;
+    cn = cs;
 // the error vector without its factor h (err_norm2 applies it once)
 #define TT_E(f) \
-    TT_MAC(T::e7, kn.f, fma(T::e6, k6.f, fma(T::e5, k5.f, fma(T::e4, k4.f, fma(T::e3, k3.f, T::e1 * k1.f)))))
+    TT_MAC(T::e7, kn.f, fma(T::e6, k6.f, fma(T::e5, k5.f, fma(T::e4, k4.f, fma(T::e3, k3.f, m.mul(k1.f, T::e1))))))
     err.r = TT_E(r);
     err.th = TT_E(th);
     err.pr = TT_E(pr);
@@ -279,14 +288,27 @@ __device__ __forceinline__ double sq3(double a, double b, double c) {
 // near 1e-75 or 1e75) takes the per-component reciprocals instead.
 // The error vector is he * e (he = h for the Runge-Kutta pairs, whose e omits
 // the step's factor h; 1 otherwise).
+// max(|a|, |b|) of two doubles that are not NaN, on the integer pipe (fmax takes
+// two FP64 issue slots: magnitudes order as their bit patterns).
+__device__ __forceinline__ double max_abs(double a, double b) {
+    const unsigned long long x = (unsigned long long)__double_as_longlong(a) & 0x7fffffffffffffffull;
+    const unsigned long long y = (unsigned long long)__double_as_longlong(b) & 0x7fffffffffffffffull;
+    return __longlong_as_double((long long)max(x, y));
+}
+
+// (yn may hold a NaN or an infinity only where the caller then ends the ray,
+// whatever the norm.)  For IntMul: the tolerances lie in 2^+-47 (the caller's
+// condition), so every scale factor is at least 2^-47, and those of r and p_r
+// are bounded by the flow's checks of yn; he is checked by rk_step64.
+template <class Mul>
 __device__ __forceinline__ double err_norm2(const State& y, const State& yn, const State& e,
-                                            double atol, double rtol, double he) {
-    const double s0 = fma(rtol, fmax(fabs(y.r), fabs(yn.r)), atol);
-    const double s1 = fma(rtol, fmax(fabs(y.th), fabs(yn.th)), atol);
-    const double s2 = fma(rtol, fmax(fabs(y.pr), fabs(yn.pr)), atol);
-    const double s3 = fma(rtol, fmax(fabs(y.pth), fabs(yn.pth)), atol);
-    const double p01 = s0 * s1, p23 = s2 * s3;
-    const double pp = p01 * p23;
+                                            double atol, double rtol, double he, Mul& m) {
+    const double s0 = fma(rtol, max_abs(y.r, yn.r), atol);
+    const double s1 = fma(rtol, max_abs(y.th, yn.th), atol);
+    const double s2 = fma(rtol, max_abs(y.pr, yn.pr), atol);
+    const double s3 = fma(rtol, max_abs(y.pth, yn.pth), atol);
+    const double p01 = m.chk(s0, s1), p23 = m.chk(s2, s3);
+    const double pp = m.mul(p01, p23);
     // outside [2^-930, 2^930] (the exponent field, on the integer pipe)
     const int ex = (__double2hiint(pp) >> 20) & 0x7ff;
     if (ex < 1023 - 930 || ex > 1023 + 930) {
@@ -297,8 +319,8 @@ __device__ __forceinline__ double err_norm2(const State& y, const State& yn, con
     }
     double inv;
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(inv) : "d"(pp));
-    inv = fma(inv, fma(-pp, inv, 1.0), inv) * he;
-    const double i01 = inv * p23, i23 = inv * p01;   // he/(s0 s1), he/(s2 s3)
+    inv = m.mul(fma(inv, fma(-pp, inv, 1.0), inv), he);
+    const double i01 = m.mul(inv, p23), i23 = m.mul(inv, p01);   // he/(s0 s1), he/(s2 s3)
     const double q0 = (e.r * s1) * i01, q1 = (e.th * s0) * i01;
     const double q2 = (e.pr * s3) * i23, q3 = (e.pth * s2) * i23;
     return 0.25 * fma(q3, q3, fma(q2, q2, fma(q1, q1, q0 * q0)));
@@ -911,6 +933,24 @@ __device__ __forceinline__ void note_crossing(Lane& L, const State& y, const Sol
     L.pend = true;
 }
 
+// A closed-form Kerr step attempt with plain FP64 products, out of line (the few
+// attempts whose products the integer pipes do not take).
+struct Step64 {
+    State yn, kn;
+    double Hn, sn, cn, err2;
+};
+
+template <int METHOD>
+__device__ __noinline__ Step64 plain_step64(const ImageDesc* d, KerrK kk, RayConst R, State y, State k1, double h,
+                                            double s0, double c0, double atol, double rtol) {
+    Step64 o;
+    State e;
+    FpMul m;
+    rk_step64<0, METHOD>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, e, s0, c0, o.sn, o.cn, m);
+    o.err2 = err_norm2(y, o.yn, e, atol, rtol, h, m);
+    return o;
+}
+
 // One FP64 step attempt; returns the termination code or -1 if the ray continues.
 template <int METRIC, int PREC, int METHOD = 0>
 __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
@@ -919,16 +959,37 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
     const double hmin = (sol.h_min > 0.0) ? sol.h_min : 1e-14 * fmax(1.0, fabs(L.lam));
     if (lt_pos(L.h, hmin)) return 3;
     State yn, kn, e;
-    double Hn, sn = L.s0, cn = L.c0;
+    double Hn, sn = L.s0, cn = L.c0, err2;
     if constexpr (METHOD == 4) {
         verlet_step64<METRIC>(d, L.kk, L.R, L.y, L.k1, L.h, yn, kn, Hn);
+        err2 = 0.0;                            // fixed step, always accepted
     } else if constexpr (METHOD == 3) {
+        FpMul m;
         gbs_step64<METRIC>(d, L.kk, L.R, L.y, L.k1, L.h, yn, kn, Hn, e);
+        err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, 1.0, m);
+    } else if constexpr (METRIC == 0 && PREC == 0) {
+        // products on the integer pipes (the FP64 unit, 87 % busy, was the bound:
+        // 258.3 -> 177.7 ms for the 1024^2 disk, issue 8 -> 22 %, the FP64 unit still
+        // 84 % busy with 2/3 of the instructions); where their operands leave the
+        // checked range (a ray in the equatorial plane, a stage inside the horizon)
+        // the attempt is made again with plain products
+        IntMul m;
+        rk_step64<METRIC, METHOD>(d, L.kk, L.R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
+        err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
+        if (!(m.ok() && sol.int_mul)) {
+            const Step64 o = plain_step64<METHOD>(&d, L.kk, L.R, L.y, L.k1, L.h, L.s0, L.c0, sol.atol, sol.rtol);
+            yn = o.yn;
+            kn = o.kn;
+            Hn = o.Hn;
+            sn = o.sn;
+            cn = o.cn;
+            err2 = o.err2;
+        }
     } else {
-        rk_step64<METRIC, METHOD>(d, L.kk, L.R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, &sn, &cn);
+        FpMul m;
+        rk_step64<METRIC, METHOD>(d, L.kk, L.R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
+        err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
     }
-    // Verlet: fixed step, always accepted
-    const double err2 = (METHOD == 4) ? 0.0 : err_norm2(L.y, yn, e, sol.atol, sol.rtol, METHOD == 3 ? 1.0 : L.h);
     if (nan_bits(err2) | nonfinite_bits(yn.r) | nonfinite_bits(yn.th) | nonfinite_bits(yn.pr) |
         nonfinite_bits(yn.pth))
         return 4;
@@ -948,7 +1009,7 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
         L.k1 = kn;
         L.s0 = sn;
         L.c0 = cn;
-        L.hmax = fmax(L.hmax, fabs(Hn));
+        if (!nan_bits(Hn)) L.hmax = max_abs(L.hmax, Hn);
         if (lt_pos(yn.r, d.r_capture)) return 1;
         if (lt_pos(d.r_escape, yn.r)) return 0;
         if constexpr (METHOD == 3) {
@@ -1068,7 +1129,8 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
         y64n = State{L.y.r + (double)inc.r, L.y.th + (double)inc.th, L.y.pr + (double)inc.pr,
                      L.y.pth + (double)inc.pth};
         const State e64 = State{(double)TT_E(r), (double)TT_E(th), (double)TT_E(pr), (double)TT_E(pth)};
-        err64 = err_norm2(L.y, y64n, e64, sol.atol, sol.rtol, 1.0);
+        FpMul m;
+        err64 = err_norm2(L.y, y64n, e64, sol.atol, sol.rtol, 1.0, m);
         err2 = nan_bits(err64) ? __int_as_float(0x7fffffff) : (err64 <= 1.0 ? 0.0f : 2.0f);
     } else {
         const float atol = (float)sol.atol, rtol = (float)sol.rtol;
