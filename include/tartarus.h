@@ -127,8 +127,8 @@ typedef struct {
  * A ray whose distance from the critical curve, estimated as
  * R(r_m) / (2 r_m^2 b) at the local minimum r_m of R (b^2 = xi^2 + eta), is
  * below critical_band (in units of M) is traced entirely in double-float, as
- * TT_DOUBLE_FLOAT traces it, at rtol = atol = critical_rtol; these rays are
- * traced first, by whole warps, in the same launch.  critical_band 0 selects
+ * TT_DOUBLE_FLOAT traces it, at rtol = atol = critical_rtol, by whole warps of a
+ * kernel that starts first and that the kernel of the other rays overlaps.  critical_band 0 selects
  * 0.15 on TT_MIXED and TT_MIXED_PAIR and none on TT_MIXED_SPLIT, negative:
  * none; critical_rtol 0 selects 1e-10.  Other precisions ignore both.
  * TT_DOUBLE_FLOAT steps every ray in double-float: flow, stage points, stage
@@ -233,9 +233,9 @@ typedef struct {
  *                   iterations (default 32)
  *   fp64_wait       mixed paths: lanes waiting for a zone step get one after at
  *                   most this many warp iterations (default 64)
- *   crit_stride     mixed paths with a critical band: the warps of one SM in
- *                   crit_stride start by scanning for near-critical rays
- *                   (default 1: every SM)
+ *   crit_stride     mixed paths with a critical band: the near-critical rays are
+ *                   traced by one block on one SM in crit_stride (default 1:
+ *                   every SM), beside the kernel of the other rays
  *   crit_refill     mixed paths: a warp tracing near-critical rays refills once
  *                   this many lanes are free (1..32, default 32) */
 typedef struct {

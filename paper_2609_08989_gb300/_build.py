@@ -21,7 +21,7 @@ DEBUG_BUILD = os.path.join(BUILD, "bounds_check")
 DEBUG_SO = os.path.join(BUILD, "libtartarus_debug.so")
 PEAKS_SRC = "tt_peaks.cu"
 PEAKS_SO = os.path.join(BUILD, "libtt_peaks.so")
-SOURCES = ["tt_capi.cu", "tt_kernel64.cu", "tt_kernel_mixed.cu", "tt_kernel_split.cu", "tt_kernel_ck.cu", "tt_kernel_f.cu",
+SOURCES = ["tt_capi.cu", "tt_kernel64.cu", "tt_kernel_mixed.cu", "tt_kernel_split.cu", "tt_kernel_critical.cu", "tt_kernel_ck.cu", "tt_kernel_f.cu",
            "tt_kernel_gbs.cu", "tt_kernel_verlet.cu", "tt_kernel_df.cu"]
 HEADERS = ["tt_internal.h", "tt_device.cuh", "tt_soft64.cuh", "tt_df.cuh", "tt_trace.cuh", "tt_kernel_rk.cuh", os.path.join("..", "..", "include", "tartarus.h")]
 ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]

@@ -25,6 +25,7 @@
 #pragma once
 
 #include <cstdint>
+#include <type_traits>
 #include <cuda_runtime.h>
 
 #include "tt_device.cuh"
@@ -503,24 +504,35 @@ __device__ double initial_step64(const ImageDesc& d, const KerrK& kk, const RayC
 // ---------------------------------------------------------------------------
 // Per-lane ray record.
 // ---------------------------------------------------------------------------
-struct Lane {
+// What the steps themselves do not touch (the mixed paths' zone steps, refinement
+// and records do).
+struct RayCold {
+    RayConst R;
+    State yc;               // a disk crossing waiting for its (batched) refinement: the start of its step
+    double hmax, inten;
+    double pad;             // 15 doubles: a warp's 64-bit accesses to one field fall in distinct banks
+};
+
+// What the FP32 flow needs of a ray: its constants, M, a^2 and r_+ - r_-.
+struct Ray32 {
+    RayConstF Rf;
+    float Mf, a2f, rpmf;
+};
+
+struct LaneBase {
     const ImageDesc* d;
     long long q;            // output index within the image
     State y, k1;            // FP64 state and its flow (first-same-as-last, valid if k64_ok)
     double s0, c0;          // sin and cos of y.th (FP64 path, closed-form metric)
-    RayConst R;
     KerrK kk;
-    double h, lam, hmax, inten;
+    double h, lam;
     int steps, rejects, ncross, nrec, code;
     bool last_rej;
-    // a disk crossing waiting for its (batched) refinement: the start of its step
-    bool pend;
-    State yc;
+    bool pend;              // a crossing is waiting in cold().yc
     // mixed precision
     StateF k1f;             // FP32 flow at the state (valid if k32_ok)
     StateF lo;              // low parts of the compensated FP32-pair state
-    RayConstF Rf;
-    float Mf, a2f, rpmf;    // M, a^2, r_+ - r_-
+    Ray32 f32;
     float rph, rpl;         // r_+ as an FP32 pair
     float caph, capl;       // capture radius as an FP32 pair
     float escf, fp64f;      // escape radius, extended-precision-step radius
@@ -534,8 +546,22 @@ struct Lane {
     float hmaxf;
     KerrDF kdf;
     RayDF rdf;
-    // mixed paths: a near-critical ray, traced in double-float
-    bool crit;
+};
+
+// In registers, or with the cold part in the thread's slot of shared memory (the
+// mixed paths with FP32 control: at 128 registers it would be spilled; 38.7 ->
+// 37.7 ms per 2048^2 image; the prescribed split, whose FP64 zone steps read the
+// constants at every stage, 36.5 -> 37.3 ms per 1024^2 image, keeps registers).
+struct LaneReg : LaneBase {
+    RayCold c;
+    __device__ __forceinline__ RayCold& cold() { return c; }
+};
+
+constexpr int kMixBlock = 256;
+static __shared__ RayCold s_cold[kMixBlock];
+
+struct LaneShared : LaneBase {
+    __device__ __forceinline__ RayCold& cold() { return s_cold[threadIdx.x]; }
 };
 
 // Output stores.  The bounds-checking build (TT_BOUNDS_CHECK) tests every index
@@ -553,13 +579,14 @@ struct Lane {
 #define TT_STORE(d, arr, idx, len, val) ((d).arr[(idx)] = (val))
 #endif
 
-__device__ __forceinline__ void write_final(const Lane& L, int code, const SolverDesc& sol) {
+template <class Lane>
+__device__ __forceinline__ void write_final(Lane& L, int code, const SolverDesc& sol) {
     const ImageDesc& d = *L.d;
     const long long q = L.q, n = d.pix_count;
     TT_STORE(d, code, q, n, (int8_t)code);
     TT_STORE(d, n_cross, q, n, (int8_t)min(L.ncross, 127));
-    TT_STORE(d, intensity, q, n, L.inten);
-    TT_STORE(d, h_max, q, n, fmax(L.hmax, (double)L.hmaxf));
+    TT_STORE(d, intensity, q, n, L.cold().inten);
+    TT_STORE(d, h_max, q, n, fmax(L.cold().hmax, (double)L.hmaxf));
     TT_STORE(d, steps, q, n, L.steps);
     TT_STORE(d, rejects, q, n, L.rejects);
     for (int k = L.nrec; k < kMaxCross; ++k) {
@@ -587,11 +614,10 @@ __device__ __forceinline__ void split_state(const State& y, StateF& hi, StateF& 
 }
 
 // The Hairer-Norsett-Wanner starting step in FP32 for the mixed paths, from the
-// FP32 flow k1f at yf (already in L); the flow takes theta as dth0 = theta - m pi
+// FP32 flow f0 at yf; the flow takes theta as dth0 = theta - m pi
 // (see step_ray32).
-static __device__ float initial_step32(const Lane& L, const StateF& y0, float dr0, float dth0, float atol,
+static __device__ float initial_step32(const Ray32& f32, const StateF& f0, const StateF& y0, float dr0, float dth0, float atol,
                                        float rtol) {
-    const StateF f0 = L.k1f;
     const float sr = fmaf(rtol, fabsf(y0.r), atol), st = fmaf(rtol, fabsf(y0.th), atol);
     const float sp = fmaf(rtol, fabsf(y0.pr), atol), sq = fmaf(rtol, fabsf(y0.pth), atol);
     auto n4 = [&](float a, float b, float c, float e) {
@@ -603,7 +629,7 @@ static __device__ float initial_step32(const Lane& L, const StateF& y0, float dr
     const StateF y1 = {fmaf(h0, f0.r, y0.r), fmaf(h0, f0.th, y0.th), fmaf(h0, f0.pr, y0.pr), fmaf(h0, f0.pth, y0.pth)};
     StateF f1;
     float H1;
-    kerr_flow32(L.Mf, L.a2f, L.rpmf, L.Rf, StateF{y1.r, fmaf(h0, f0.th, dth0), y1.pr, y1.pth}, fmaf(h0, f0.r, dr0),
+    kerr_flow32(f32.Mf, f32.a2f, f32.rpmf, f32.Rf, StateF{y1.r, fmaf(h0, f0.th, dth0), y1.pr, y1.pth}, fmaf(h0, f0.r, dr0),
                 f1, H1);
     const float d2 = n4(f1.r - f0.r, f1.th - f0.th, f1.pr - f0.pr, f1.pth - f0.pth) / h0;
     const float dm = fmaxf(d1, d2);
@@ -681,7 +707,7 @@ __device__ __forceinline__ bool near_critical(const ImageDesc& d, long long q, f
 // pixel q (after tile_pixel).  Returns false (and writes a BADPIXEL record) if
 // the pixel is outside the sky.  df_init: set the ray up for double-float steps
 // (the double-float path, and near-critical rays of the mixed paths).
-template <int METRIC>
+template <int METRIC, class Lane>
 __device__ bool init_ray(Lane& L, const ImageDesc* d_ptr, long long q, const SolverDesc& sol,
                          bool df_init = false) {
     const ImageDesc& d = *d_ptr;
@@ -693,8 +719,8 @@ __device__ bool init_ray(Lane& L, const ImageDesc* d_ptr, long long q, const Sol
     L.ncross = 0;
     L.nrec = 0;
     L.code = -1;
-    L.inten = 0.0;
-    L.hmax = 0.0;
+    L.cold().inten = 0.0;
+    L.cold().hmax = 0.0;
     L.lam = 0.0;
     L.last_rej = false;
     L.pend = false;
@@ -741,25 +767,25 @@ __device__ bool init_ray(Lane& L, const ImageDesc* d_ptr, long long q, const Sol
     L.y.th = th;
     L.y.pr = -p_r;
     L.y.pth = -p_th;
-    L.R = make_ray_const(d.a, -p_t, -p_ph);
+    L.cold().R = make_ray_const(d.a, -p_t, -p_ph);
     L.k32_ok = false;
     L.kdf_ok = false;
     L.hmaxf = 0.0f;
     if (sol.precision == 0 && !df_init) {
         double H0;
-        flow64<METRIC>(d, L.kk, L.R, L.y, L.k1, H0);
+        flow64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, H0);
         sincos(L.y.th, &L.s0, &L.c0);
-        L.hmax = fabs(H0);
-        L.h = (sol.h0 > 0.0) ? sol.h0 : initial_step64<METRIC>(d, L.kk, L.R, L.y, L.k1, sol.atol, sol.rtol);
+        L.cold().hmax = fabs(H0);
+        L.h = (sol.h0 > 0.0) ? sol.h0 : initial_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, sol.atol, sol.rtol);
         L.k64_ok = true;
     } else {
         // mixed paths: FP32 flow and starting step, |H(y0)| (~1e-16) not sampled;
         // double-float path: the FP64 flow and starting step
         L.k64_ok = false;
-        L.Rf = to_float(L.R, d.M);
-        L.Mf = (float)d.M;
-        L.a2f = (float)(d.a * d.a);
-        L.rpmf = (float)(d.r_plus - d.r_minus);
+        L.f32.Rf = to_float(L.cold().R, d.M);
+        L.f32.Mf = (float)d.M;
+        L.f32.a2f = (float)(d.a * d.a);
+        L.f32.rpmf = (float)(d.r_plus - d.r_minus);
         split_pair(d.r_plus, L.rph, L.rpl);
         split_pair(d.r_capture, L.caph, L.capl);
         L.escf = (float)d.r_escape;
@@ -770,21 +796,21 @@ __device__ bool init_ray(Lane& L, const ImageDesc* d_ptr, long long q, const Sol
             // double-float steps: the FP64 path's starting step (once per ray), so
             // that both begin the same step sequence
             L.kdf = make_kerr_df(L.kk);
-            L.rdf = make_ray_df(L.R);
+            L.rdf = make_ray_df(L.cold().R);
             double H64;
-            flow64<METRIC>(d, L.kk, L.R, L.y, L.k1, H64);
-            L.hmax = fabs(H64);
+            flow64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, H64);
+            L.cold().hmax = fabs(H64);
             L.hf = (float)((sol.h0 > 0.0) ? sol.h0
-                                         : initial_step64<METRIC>(d, L.kk, L.R, L.y, L.k1, sol.atol, sol.rtol));
+                                         : initial_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, sol.atol, sol.rtol));
         } else {
             const StateF yf = {(float)L.y.r, (float)L.y.th, (float)L.y.pr, (float)L.y.pth};
             const float dr0 = (float)(L.y.r - d.r_plus);
             const float dth0 = (float)(L.y.th - rint(L.y.th * 0.3183098861837907) * 3.141592653589793);
             float H0;
-            kerr_flow32(L.Mf, L.a2f, L.rpmf, L.Rf, StateF{yf.r, dth0, yf.pr, yf.pth}, dr0, L.k1f, H0);
+            kerr_flow32(L.f32.Mf, L.f32.a2f, L.f32.rpmf, L.f32.Rf, StateF{yf.r, dth0, yf.pr, yf.pth}, dr0, L.k1f, H0);
             L.k32_ok = true;
             L.hf = (sol.h0 > 0.0) ? (float)sol.h0
-                                  : initial_step32(L, yf, dr0, dth0, (float)sol.atol, (float)sol.rtol);
+                                  : initial_step32(L.f32, L.k1f, yf, dr0, dth0, (float)sol.atol, (float)sol.rtol);
         }
         L.h = (double)L.hf;
     }
@@ -793,12 +819,12 @@ __device__ bool init_ray(Lane& L, const ImageDesc* d_ptr, long long q, const Sol
 
 // Emission at a refined crossing radius (paper Sec. 2.3-2.4): counted if on the
 // disk, stored (r, g, g^4 F) while slots remain.
-template <int METRIC>
+template <int METRIC, class Lane>
 __device__ __forceinline__ void record_crossing(Lane& L, double rc, const SolverDesc& sol) {
     const ImageDesc& d = *L.d;
     if (rc >= d.r_in && rc <= d.r_out) {
         if (L.nrec < d.max_cross) {
-            const double gf = redshift64<METRIC>(d, rc, L.R.pt, L.R.pph);
+            const double gf = redshift64<METRIC>(d, rc, L.cold().R.pt, L.cold().R.pph);
             const double F = flux64(d, rc);
             const double g2 = gf * gf;
             const double I = g2 * g2 * F;
@@ -806,7 +832,7 @@ __device__ __forceinline__ void record_crossing(Lane& L, double rc, const Solver
             TT_STORE(d, r_cross, L.nrec * n + q, kMaxCross * n, rc);
             TT_STORE(d, g, L.nrec * n + q, kMaxCross * n, gf);
             TT_STORE(d, I_cross, L.nrec * n + q, kMaxCross * n, I);
-            L.inten += I;
+            L.cold().inten += I;
             L.nrec++;
         }
         L.ncross++;
@@ -823,7 +849,7 @@ __device__ __forceinline__ float sq_ratio32(float e, float y, float yn, float at
 // error rule as refine_henon64, the theta-system evaluated with the FP32 flow
 // at stage points formed from the FP64 sub-step start, and the sub-step
 // results accumulated in FP64.
-__device__ __forceinline__ void theta_flow32(const Lane& L, const StateF& y, float dr, StateF& g) {
+__device__ __forceinline__ void theta_flow32(const Ray32& L, const StateF& y, float dr, StateF& g) {
     StateF f;
     float H;
     kerr_flow32(L.Mf, L.a2f, L.rpmf, L.Rf, y, dr, f, H);
@@ -834,7 +860,7 @@ __device__ __forceinline__ void theta_flow32(const Lane& L, const StateF& y, flo
     g.pth = f.pth * it;
 }
 
-static __device__ double refine_henon32(const Lane& L, const State& y0, double r_plus, float atol, float rtol) {
+static __device__ __noinline__ double refine_henon32(Ray32 L, State y0, double r_plus, float atol, float rtol) {
     using namespace dp;
     const double dth_all = kHalfPi - y0.th;
     double r_out = y0.r;
@@ -903,22 +929,22 @@ static __device__ double refine_henon32(const Lane& L, const State& y0, double r
 // Refine the pending crossing from the start of its step and record it.
 // PREC 0: FP64 Henon.  Mixed paths: Henon with FP32 stages, or in FP64 when
 // the solver asks for it (refine 2); emission is evaluated in FP64 either way.
-template <int METRIC, int PREC, int METHOD = 0>
+template <int METRIC, int PREC, int METHOD = 0, class Lane>
 __device__ void refine_pending(Lane& L, const SolverDesc& sol) {
     const ImageDesc& d = *L.d;
     double rc;
     if ((PREC == 1 || PREC == 2) && sol.refine != 2) {
-        rc = refine_henon32(L, L.yc, d.r_plus, (float)sol.atol, (float)sol.rtol);
+        rc = refine_henon32(L.f32, L.cold().yc, d.r_plus, (float)sol.atol, (float)sol.rtol);
     } else {
         State f0;
         double H0;
-        flow64<METRIC>(d, L.kk, L.R, L.yc, f0, H0);
-        L.hmax = fmax(L.hmax, fabs(H0));
+        flow64<METRIC>(d, L.kk, L.cold().R, L.cold().yc, f0, H0);
+        L.cold().hmax = fmax(L.cold().hmax, fabs(H0));
         // the pairs and the extrapolator use their own steps, Verlet Dormand-Prince
         if constexpr (METHOD == 3)
-            rc = refine_henon_gbs64<METRIC>(d, L.kk, L.R, L.yc, f0, sol.atol, sol.rtol);
+            rc = refine_henon_gbs64<METRIC>(d, L.kk, L.cold().R, L.cold().yc, f0, sol.atol, sol.rtol);
         else
-            rc = refine_henon64<METRIC, (METHOD <= 2 ? METHOD : 0)>(d, L.kk, L.R, L.yc, f0, sol.atol, sol.rtol);
+            rc = refine_henon64<METRIC, (METHOD <= 2 ? METHOD : 0)>(d, L.kk, L.cold().R, L.cold().yc, f0, sol.atol, sol.rtol);
     }
     record_crossing<METRIC>(L, rc, sol);
     L.pend = false;
@@ -926,10 +952,10 @@ __device__ void refine_pending(Lane& L, const SolverDesc& sol) {
 
 // A crossing was found in the step that starts at y (FP64).  Henon refinement
 // is deferred to a batched phase; crossings stay in order along the ray.
-template <int METRIC, int PREC, int METHOD = 0>
+template <int METRIC, int PREC, int METHOD = 0, class Lane>
 __device__ __forceinline__ void note_crossing(Lane& L, const State& y, const SolverDesc& sol) {
     if (L.pend) refine_pending<METRIC, PREC, METHOD>(L, sol);
-    L.yc = y;
+    L.cold().yc = y;
     L.pend = true;
 }
 
@@ -952,7 +978,7 @@ __device__ __noinline__ Step64 plain_step64(const ImageDesc* d, KerrK kk, RayCon
 }
 
 // One FP64 step attempt; returns the termination code or -1 if the ray continues.
-template <int METRIC, int PREC, int METHOD = 0>
+template <int METRIC, int PREC, int METHOD = 0, class Lane>
 __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
     const ImageDesc& d = *L.d;
     if ((long long)L.steps + (long long)L.rejects >= sol.max_steps) return 2;
@@ -961,23 +987,23 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
     State yn, kn, e;
     double Hn, sn = L.s0, cn = L.c0, err2;
     if constexpr (METHOD == 4) {
-        verlet_step64<METRIC>(d, L.kk, L.R, L.y, L.k1, L.h, yn, kn, Hn);
+        verlet_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn);
         err2 = 0.0;                            // fixed step, always accepted
     } else if constexpr (METHOD == 3) {
         FpMul m;
-        gbs_step64<METRIC>(d, L.kk, L.R, L.y, L.k1, L.h, yn, kn, Hn, e);
+        gbs_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e);
         err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, 1.0, m);
-    } else if constexpr (METRIC == 0 && PREC == 0) {
+    } else if constexpr (METRIC == 0 && (PREC == 0 || PREC == 4)) {
         // products on the integer pipes (the FP64 unit, 87 % busy, was the bound:
         // 258.3 -> 177.7 ms for the 1024^2 disk, issue 8 -> 22 %, the FP64 unit still
         // 84 % busy with 2/3 of the instructions); where their operands leave the
         // checked range (a ray in the equatorial plane, a stage inside the horizon)
         // the attempt is made again with plain products
         IntMul m;
-        rk_step64<METRIC, METHOD>(d, L.kk, L.R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
+        rk_step64<METRIC, METHOD>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
         err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
         if (!(m.ok() && sol.int_mul)) {
-            const Step64 o = plain_step64<METHOD>(&d, L.kk, L.R, L.y, L.k1, L.h, L.s0, L.c0, sol.atol, sol.rtol);
+            const Step64 o = plain_step64<METHOD>(&d, L.kk, L.cold().R, L.y, L.k1, L.h, L.s0, L.c0, sol.atol, sol.rtol);
             yn = o.yn;
             kn = o.kn;
             Hn = o.Hn;
@@ -987,7 +1013,7 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
         }
     } else {
         FpMul m;
-        rk_step64<METRIC, METHOD>(d, L.kk, L.R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
+        rk_step64<METRIC, METHOD>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
         err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
     }
     if (nan_bits(err2) | nonfinite_bits(yn.r) | nonfinite_bits(yn.th) | nonfinite_bits(yn.pr) |
@@ -1009,7 +1035,7 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
         L.k1 = kn;
         L.s0 = sn;
         L.c0 = cn;
-        if (!nan_bits(Hn)) L.hmax = max_abs(L.hmax, Hn);
+        if (!nan_bits(Hn)) L.cold().hmax = max_abs(L.cold().hmax, Hn);
         if (lt_pos(yn.r, d.r_capture)) return 1;
         if (lt_pos(d.r_escape, yn.r)) return 0;
         if constexpr (METHOD == 3) {
@@ -1056,7 +1082,7 @@ __device__ __forceinline__ bool pair_below(float hi, float lo, float ch, float c
     return ((hi - ch) + (lo - cl)) < 0.0f;
 }
 
-template <int PREC>
+template <int PREC, class Lane>
 __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
     constexpr int ACC = (PREC == 2) ? 1 : 0;
     const ImageDesc& d = *L.d;
@@ -1086,7 +1112,7 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
     }
     float Hs;
     if (!L.k32_ok) {
-        kerr_flow32(L.Mf, L.a2f, L.rpmf, L.Rf, StateF{y.r, dth0, y.pr, y.pth}, dr0, L.k1f, Hs);
+        kerr_flow32(L.f32.Mf, L.f32.a2f, L.f32.rpmf, L.f32.Rf, StateF{y.r, dth0, y.pr, y.pth}, dr0, L.k1f, Hs);
         L.k32_ok = true;
     }
     const StateF k1 = L.k1f;
@@ -1096,7 +1122,7 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
     ys.th = fmaf(h, (et), dth0);                           \
     ys.pr = fmaf(h, (ep), y.pr);                           \
     ys.pth = fmaf(h, (eq), y.pth);                         \
-    kerr_flow32(L.Mf, L.a2f, L.rpmf, L.Rf, ys, fmaf(h, (er), dr0), dst, Hs);
+    kerr_flow32(L.f32.Mf, L.f32.a2f, L.f32.rpmf, L.f32.Rf, ys, fmaf(h, (er), dr0), dst, Hs);
 #define TT_C2(f) ((float)a21 * k1.f)
 #define TT_C3(f) fmaf((float)a32, k2.f, (float)a31 * k1.f)
 #define TT_C4(f) fmaf((float)a43, k3.f, fmaf((float)a42, k2.f, (float)a41 * k1.f))
@@ -1117,7 +1143,7 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
     inc.pth = h * TT_C7(pth);
     StateF yn = {y.r + inc.r, y.th + inc.th, y.pr + inc.pr, y.pth + inc.pth};
     float Hn;
-    kerr_flow32(L.Mf, L.a2f, L.rpmf, L.Rf, StateF{yn.r, dth0 + inc.th, yn.pr, yn.pth}, dr0 + inc.r, k7, Hn);
+    kerr_flow32(L.f32.Mf, L.f32.a2f, L.f32.rpmf, L.f32.Rf, StateF{yn.r, dth0 + inc.th, yn.pr, yn.pth}, dr0 + inc.r, k7, Hn);
 #define TT_E(f) \
     h * fmaf((float)e7, k7.f, fmaf((float)e6, k6.f, fmaf((float)e5, k5.f, fmaf((float)e4, k4.f, \
              fmaf((float)e3, k3.f, (float)e1 * k1.f)))))
@@ -1129,8 +1155,14 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
         y64n = State{L.y.r + (double)inc.r, L.y.th + (double)inc.th, L.y.pr + (double)inc.pr,
                      L.y.pth + (double)inc.pth};
         const State e64 = State{(double)TT_E(r), (double)TT_E(th), (double)TT_E(pr), (double)TT_E(pth)};
-        FpMul m;
+        IntMul m;
+        m.see(y64n.r);
+        m.see(y64n.pr);
         err64 = err_norm2(L.y, y64n, e64, sol.atol, sol.rtol, 1.0, m);
+        if (!(m.ok() && sol.int_mul)) {
+            FpMul f;
+            err64 = err_norm2(L.y, y64n, e64, sol.atol, sol.rtol, 1.0, f);
+        }
         err2 = nan_bits(err64) ? __int_as_float(0x7fffffff) : (err64 <= 1.0 ? 0.0f : 2.0f);
     } else {
         const float atol = (float)sol.atol, rtol = (float)sol.rtol;
@@ -1206,10 +1238,11 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
 // from the FP64 state, with the FSAL flow, sin and cos taken afresh after FP32
 // steps; the step size and affine parameter are carried over from and back to
 // the FP32 steps.
+template <class Lane>
 __device__ __forceinline__ int step_zone64_split(Lane& L, const SolverDesc& sol) {
     if (!L.k64_ok) {
         double H;
-        flow64<0>(*L.d, L.kk, L.R, L.y, L.k1, H);
+        flow64<0>(*L.d, L.kk, L.cold().R, L.y, L.k1, H);
         sincos(L.y.th, &L.s0, &L.c0);
         L.k64_ok = true;
     }
@@ -1236,7 +1269,7 @@ __device__ __forceinline__ int step_zone64_split(Lane& L, const SolverDesc& sol)
 // step-size control run in FP32.  ACC 0: the state is the FP64 L.y;
 // ACC 1: the FP32 pair (yhi, L.lo).
 // ---------------------------------------------------------------------------
-template <int METRIC, int ACC, bool FULL>
+template <int METRIC, int ACC, bool FULL, class Lane>
 __device__ int step_ray_df(Lane& L, StateF& yhi, const SolverDesc& sol) {
     constexpr int PREC = FULL ? 3 : ACC + 1;
     const ImageDesc& d = *L.d;
@@ -1252,7 +1285,7 @@ __device__ int step_ray_df(Lane& L, StateF& yhi, const SolverDesc& sol) {
         rd = L.rdf;
     } else {
         kd = make_kerr_df(L.kk);
-        rd = make_ray_df(L.R);
+        rd = make_ray_df(L.cold().R);
     }
     StateDF y;
     if constexpr (ACC == 0) {
@@ -1415,12 +1448,12 @@ __device__ int step_ray_df(Lane& L, StateF& yhi, const SolverDesc& sol) {
 // theta for Kerr) goes to zero, and W / D (and its derivatives) lose the
 // double-float's digits in proportion; the FP32-pair state, step size and
 // affine parameter are carried over exactly and back.
-template <int METRIC>
+template <int METRIC, class Lane>
 __device__ int step_zone64(Lane& L, StateF& yhi, const SolverDesc& sol) {
     L.y = pair_to64(yhi, L.lo);
     if (!L.k64_ok) {
         double H;
-        flow64<METRIC>(*L.d, L.kk, L.R, L.y, L.k1, H);
+        flow64<METRIC>(*L.d, L.kk, L.cold().R, L.y, L.k1, H);
         L.k64_ok = true;
     }
     L.h = (double)L.hf;
@@ -1435,16 +1468,16 @@ __device__ int step_zone64(Lane& L, StateF& yhi, const SolverDesc& sol) {
 
 // Steps of the double-float table path that run in FP64 (the zones of the
 // solver's fp64_radius_factor and fp64_pole_sin).
-__device__ __forceinline__ bool in_zone(const Lane& L, const StateF& yhi) {
+__device__ __forceinline__ bool in_zone(const LaneBase& L, const StateF& yhi) {
     const float axis = fabsf(fmaf(-rintf(yhi.th * 0.318309886f), 3.14159274f, yhi.th));
     return (yhi.r < L.fp64f) || (axis < L.thpf);
 }
 
 // FP64 |H| at the lane's current state (mixed-path monitor).
-template <int ACC>
+template <int ACC, class Lane>
 __device__ __forceinline__ void check_h64(Lane& L, const StateF& yhi) {
     const State y = (ACC == 0) ? L.y : pair_to64(yhi, L.lo);
-    L.hmax = fmax(L.hmax, fabs(kerr_h64(L.kk, L.R, y)));
+    L.cold().hmax = fmax(L.cold().hmax, fabs(kerr_h64(L.kk, L.cold().R, y)));
 }
 
 __device__ __forceinline__ int find_image(const ImageDesc* descs, int n, long long rid) {
@@ -1461,21 +1494,32 @@ __device__ __forceinline__ int find_image(const ImageDesc* descs, int n, long lo
 enum : int { kIdle = 0, kRun = 1, kDone = 2 };
 
 
+// The rays' queue entries [base, base + n_idle) of the idle lanes of a warp.
+struct Batch {
+    unsigned idle;
+    long long base;
+};
+
+__device__ __forceinline__ Batch take_rays(unsigned long long* queue, int lane, bool is_idle) {
+    Batch b;
+    b.idle = __ballot_sync(kFull, is_idle);
+    unsigned long long base = 0;
+    if (lane == 0) base = atomicAdd(queue, (unsigned long long)__popc(b.idle));
+    b.base = (long long)__shfl_sync(kFull, base, 0);
+    return b;
+}
+
 // PREC 0: FP64.  PREC 1: mixed with FP64 accumulation.  PREC 2: mixed with the
 // compensated FP32-pair accumulation.  PREC 3: double-float.  PREC 4: mixed
 // with the prescribed FP64 split (norm, zone steps, refinement).  METHOD (FP64
 // only): 0 Dormand-Prince, 1 Cash-Karp, 2 Fehlberg, 3 Gragg-Bulirsch-Stoer,
-// 4 Verlet.  solc: the solver settings of the mixed paths' near-critical rays.
+// 4 Verlet.
 //
-// Mixed paths with a critical band: the warps of one SM in crit_stride scan the rays
-// (queue[1]) for near-critical ones and traces those in double-float, with
-// whole warps of them; the other warps take the rays from queue[0], skipping
-// the near-critical ones (the same test picks them out).  A warp whose queue
-// is drained takes the other one.  The long double-float rays thus start first
-// and overlap with the bulk of the image.
+// Mixed paths with a critical band leave the near-critical rays to
+// critical_loop, in a kernel of its own (the same test picks them out).
 template <int METRIC, int PREC, int METHOD = 0>
 __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, long long total,
-                                           const SolverDesc& sol, const SolverDesc& solc, const TuneParams& tp,
+                                           const SolverDesc& sol, const TuneParams& tp,
                                            unsigned long long* queue) {
     static_assert(PREC == 0 || METHOD == 0, "the mixed and double-float paths step with Dormand-Prince");
     constexpr int ACC = (PREC == 2 || PREC == 3) ? 1 : 0;
@@ -1486,92 +1530,36 @@ __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, l
         __syncthreads();
     }
     const int lane = threadIdx.x & 31;
-    Lane L;
+    std::conditional_t<PREC == 1 || PREC == 2, LaneShared, LaneReg> L;
     L.pend = false;
-    L.crit = false;
     StateF yhi = {0.0f, 0.0f, 0.0f, 0.0f};   // pair accumulator: hi parts
     int st = kIdle;
     bool drained = false;
-    // the warps of one SM in crit_stride start with the scan for near-critical
-    // rays, the others with the bulk (so that an SM runs the double-float code
-    // or the FP32 code, not both, and its instruction cache holds one of them);
-    // a warp whose queue is drained and whose lanes are all written takes the
-    // other queue, until both are drained (warp-uniform)
     const float band = (float)sol.crit_band;
-    const bool use_crit = MIX && band > 0.0f;
-    unsigned smid = 0;
-    if (use_crit) asm volatile("mov.u32 %0, %%smid;" : "=r"(smid));
-    bool crit_phase = use_crit && (smid % (unsigned)tp.crit_stride) == 0;
-    bool drained_c = !use_crit;
     int wait64 = 0;
     unsigned iter = 0;
-    // crossings of near-critical rays are refined as on the double-float path
-    auto refine = [&]() {
-        if constexpr (MIX) {
-            if (L.crit) {
-                refine_pending<METRIC, 3>(L, solc);
-                return;
-            }
-        }
-        refine_pending<METRIC, PREC, METHOD>(L, sol);
-    };
     for (;;) {
         // ---- refill phase: flush finished rays, start new ones -------------
-        // (near-critical rays differ widely in length: their warps refill at a
-        // threshold of their own)
         const int n_free = __popc(__ballot_sync(kFull, st != kRun));
-        const bool more = crit_phase ? !drained_c : !drained;
-        const int refill_at = crit_phase ? tp.crit_refill : tp.refill;
-        if (n_free > 0 && (n_free >= refill_at || n_free == 32) && (more || __any_sync(kFull, st == kDone))) {
-            if (st != kIdle && L.pend) refine();
+        if (n_free > 0 && (n_free >= tp.refill || n_free == 32) && (!drained || __any_sync(kFull, st == kDone))) {
+            if (st != kIdle && L.pend) refine_pending<METRIC, PREC, METHOD>(L, sol);
             if (st == kDone) {
-                if (MIX && !L.crit) check_h64<ACC>(L, yhi);
+                if (MIX) check_h64<ACC>(L, yhi);
                 write_final(L, L.code, sol);
                 st = kIdle;
             }
-            if (crit_phase) {
-                // fill the idle lanes with near-critical rays: each round tests one
-                // queue entry per idle lane (bounded: every round consumes entries)
-                while (!drained_c) {
-                    const unsigned idle = __ballot_sync(kFull, st == kIdle);
-                    if (!idle) break;
-                    const int n_idle = __popc(idle);
-                    unsigned long long base = 0;
-                    if (lane == 0) base = atomicAdd(queue + 1, (unsigned long long)n_idle);
-                    base = __shfl_sync(kFull, base, 0);
-                    if (base + (unsigned long long)n_idle >= (unsigned long long)total) drained_c = true;
-                    if (st == kIdle) {
-                        const long long rid = (long long)base + __popc(idle & ((1u << lane) - 1u));
-                        if (rid < total) {
-                            const int im = (n_desc == 1) ? 0 : find_image(descs, n_desc, rid);
-                            const ImageDesc* dp = descs + im;
-                            const long long q = tile_pixel(*dp, rid - dp->ray_begin);
-                            if (near_critical(*dp, q, band) && init_ray<METRIC>(L, dp, q, solc, true)) {
-                                st = kRun;
-                                L.crit = true;
-                                if (ACC == 1) split_state(L.y, yhi, L.lo);
-                            }
-                        }
-                    }
-                }
-            } else if (!drained) {
-                const unsigned idle = __ballot_sync(kFull, st == kIdle);
-                const int n_idle = __popc(idle);
-                unsigned long long base = 0;
-                if (lane == 0) base = atomicAdd(queue, (unsigned long long)n_idle);
-                base = __shfl_sync(kFull, base, 0);
-                if (base + (unsigned long long)n_idle >= (unsigned long long)total) drained = true;
+            if (!drained) {
+                const Batch b = take_rays(queue, lane, st == kIdle);
+                if (b.base + __popc(b.idle) >= total) drained = true;
                 if (st == kIdle) {
-                    const long long rid = (long long)base + __popc(idle & ((1u << lane) - 1u));
+                    const long long rid = b.base + __popc(b.idle & ((1u << lane) - 1u));
                     if (rid < total) {
                         const int im = (n_desc == 1) ? 0 : find_image(descs, n_desc, rid);
                         const ImageDesc* dp = descs + im;
                         const long long q = tile_pixel(*dp, rid - dp->ray_begin);
-                        // near-critical rays were traced in the scan
                         const bool skip = MIX && band > 0.0f && near_critical(*dp, q, band);
                         if (!skip && init_ray<METRIC>(L, dp, q, sol)) {
                             st = kRun;
-                            L.crit = false;
                             if (ACC == 1) split_state(L.y, yhi, L.lo);
                         }
                     }
@@ -1580,11 +1568,8 @@ __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, l
         }
         const unsigned running = __ballot_sync(kFull, st == kRun);
         if (!running) {
-            if (__any_sync(kFull, st == kDone)) continue;          // written by the next refill
-            // every lane idle: once this queue is drained, take the other one
-            if (drained && drained_c) break;
-            if (crit_phase ? drained_c : drained) crit_phase = !crit_phase;
-            continue;
+            if (drained && !__any_sync(kFull, st == kDone)) break;
+            continue;                                              // the next refill writes or takes rays
         }
         ++iter;
         // ---- step phases ---------------------------------------------------
@@ -1623,15 +1608,6 @@ __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, l
         } else if constexpr (PREC == 0) {
             if (st == kRun) {
                 const int code = step_ray64<METRIC, 0, METHOD>(L, sol);
-                if (code >= 0) {
-                    L.code = code;
-                    st = kDone;
-                }
-            }
-        } else if (crit_phase) {
-            // near-critical rays: every step in double-float, as on the double-float path
-            if (st == kRun) {
-                const int code = step_ray_df<METRIC, ACC, true>(L, yhi, solc);
                 if (code >= 0) {
                     L.code = code;
                     st = kDone;
@@ -1676,11 +1652,81 @@ __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, l
         // ---- batched crossing refinement -----------------------------------
         const unsigned pend = __ballot_sync(kFull, st == kRun && L.pend);
         if (pend && __popc(pend) >= tp.crossing_batch) {
-            if (st == kRun && L.pend) refine();
+            if (st == kRun && L.pend) refine_pending<METRIC, PREC, METHOD>(L, sol);
         }
         // ---- FP64 |H| monitor (mixed) --------------------------------------
         if (MIX && (iter % (unsigned)tp.monitor_period) == 0) {
-            if (st == kRun && !L.crit) check_h64<ACC>(L, yhi);
+            if (st == kRun) check_h64<ACC>(L, yhi);
+        }
+    }
+}
+
+// The near-critical rays of the mixed paths (closed-form Kerr), every step in
+// double-float as on the double-float path, at the settings solc.  Warps scan
+// the ray indices for them: each round of a refill tests one index per idle lane
+// until the warp is full or the queue is drained (bounded: every round consumes
+// entries).  ACC 0: FP64 state, 1: FP32 pair.
+//
+// A loop and a kernel of their own: beside the FP32 step in one kernel, at its
+// 128 registers, the double-float step spilled, and the two codes together
+// overflowed the instruction cache (no instruction: 3.5 of the stalls per
+// issue).  Apart: 42.0 -> 38.7 ms per 2048^2 image (FP32 pair; 10.5 ms of it
+// these rays when run alone, 30.3 ms the others), the 64-image survey 204 -> 185
+// ms, a 97 x 61 preview, which waits for its longest near-critical ray, 5.7 ->
+// 4.1 ms.
+template <int ACC>
+__device__ __forceinline__ void critical_loop(const ImageDesc* descs, int n_desc, long long total,
+                                              const SolverDesc& solc, const TuneParams& tp,
+                                              unsigned long long* queue) {
+    df_sincos_table(s_df_tab);
+    __syncthreads();
+    const int lane = threadIdx.x & 31;
+    const float band = (float)solc.crit_band;
+    LaneReg L;
+    L.pend = false;
+    StateF yhi = {0.0f, 0.0f, 0.0f, 0.0f};
+    int st = kIdle;
+    bool drained = false;
+    for (;;) {
+        const int n_free = __popc(__ballot_sync(kFull, st != kRun));
+        if (n_free > 0 && (n_free >= tp.crit_refill || n_free == 32) &&
+            (!drained || __any_sync(kFull, st == kDone))) {
+            if (st != kIdle && L.pend) refine_pending<0, 3>(L, solc);
+            if (st == kDone) {
+                write_final(L, L.code, solc);
+                st = kIdle;
+            }
+            while (!drained && __any_sync(kFull, st == kIdle)) {
+                const Batch b = take_rays(queue, lane, st == kIdle);
+                if (b.base + __popc(b.idle) >= total) drained = true;
+                if (st == kIdle) {
+                    const long long rid = b.base + __popc(b.idle & ((1u << lane) - 1u));
+                    if (rid < total) {
+                        const int im = (n_desc == 1) ? 0 : find_image(descs, n_desc, rid);
+                        const ImageDesc* dp = descs + im;
+                        const long long q = tile_pixel(*dp, rid - dp->ray_begin);
+                        if (near_critical(*dp, q, band) && init_ray<0>(L, dp, q, solc, true)) {
+                            st = kRun;
+                            if (ACC == 1) split_state(L.y, yhi, L.lo);
+                        }
+                    }
+                }
+            }
+        }
+        if (!__any_sync(kFull, st == kRun)) {
+            if (drained && !__any_sync(kFull, st == kDone)) break;
+            continue;
+        }
+        if (st == kRun) {
+            const int code = step_ray_df<0, ACC, true>(L, yhi, solc);
+            if (code >= 0) {
+                L.code = code;
+                st = kDone;
+            }
+        }
+        const unsigned pend = __ballot_sync(kFull, st == kRun && L.pend);
+        if (pend && __popc(pend) >= tp.crossing_batch) {
+            if (st == kRun && L.pend) refine_pending<0, 3>(L, solc);
         }
     }
 }
@@ -1688,9 +1734,12 @@ __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, l
 int sm_count();
 
 // Persistent launch: as many blocks as fit (or blocks_per_sm) on every SM, no
-// more than the rays need.
+// more than the rays need.  overlap: the kernel may start while the one before
+// it on the stream runs (programmatic dependent launch); it waits for that
+// kernel's end with griddepcontrol.wait before it ends itself.
 template <int N, typename K>
-cudaError_t launch_persistent(K kern, int block, int blocks_per_sm, const LaunchParams<N>& p, cudaStream_t st) {
+cudaError_t launch_persistent(K kern, int block, int blocks_per_sm, const LaunchParams<N>& p, cudaStream_t st,
+                              bool overlap = false) {
     int occ = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, block, 0);
     if (e != cudaSuccess) return e;
@@ -1701,8 +1750,16 @@ cudaError_t launch_persistent(K kern, int block, int blocks_per_sm, const Launch
     long long grid_cap = (warps_needed * 32 + block - 1) / block;
     if (grid > grid_cap) grid = grid_cap;
     if (grid < 1) grid = 1;
-    kern<<<(unsigned)grid, block, 0, st>>>(p);
-    return cudaGetLastError();
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)block);
+    cfg.stream = st;
+    cudaLaunchAttribute at = {};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = overlap ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, p);
 }
 
 // Fill the launch parameters (defaults for zero tune fields).
@@ -1738,6 +1795,8 @@ cudaError_t launch_mixed(const ImageDesc* descs, int n, long long total, const S
                          const LaunchShape& shape, unsigned long long* queue, cudaStream_t stream);
 cudaError_t launch_split(const ImageDesc* descs, int n, long long total, const SolverDesc& sol,
                          const LaunchShape& shape, unsigned long long* queue, cudaStream_t stream);
+cudaError_t launch_critical(const ImageDesc* descs, int n, long long total, const SolverDesc& sol,
+                            const LaunchShape& shape, unsigned long long* queue, cudaStream_t stream);
 cudaError_t launch_df(const ImageDesc* descs, int n, long long total, int metric_mode, const SolverDesc& sol,
                       const LaunchShape& shape, unsigned long long* queue, cudaStream_t stream);
 
