@@ -434,7 +434,9 @@ __device__ __forceinline__ void lower64(const ImageDesc& d, double r, double th,
 
 // ---------------------------------------------------------------------------
 // Page-Thorne flux (paper Sec. 2.3, prefactor as printed) with the host-resolved
-// roots and coefficients; zero inside the ISCO.
+// roots and coefficients; zero inside the ISCO.  (Emission is written with
+// operations that the compiler does not contract, so that it rounds alike at
+// every place it is inlined, in every build.)
 // ---------------------------------------------------------------------------
 __device__ __forceinline__ double flux64(const ImageDesc& d, double r) {
     double x = sqrt(r / d.M);
@@ -443,9 +445,11 @@ __device__ __forceinline__ double flux64(const ImageDesc& d, double r) {
 #pragma unroll
     for (int i = 0; i < 3; ++i)
         if (d.fcoef[i] != 0.0) sum = fma(d.fcoef[i], log(x - d.fxr[i]) - d.flog0[i], sum);
-    double br = x - d.fx0 - 1.5 * d.fa * log(x / d.fx0) - sum;
+    const double l = __dmul_rn(1.5 * d.fa, log(x / d.fx0));
+    double br = __dsub_rn(__dsub_rn(x - d.fx0, l), sum);
     double x2 = x * x;
-    double pref = 3.0 / (2.0 * x2 * x2 * (x2 * x - 3.0 * x + 2.0 * d.fa));
+    const double cubic = __dadd_rn(__dsub_rn(__dmul_rn(x2, x), __dmul_rn(3.0, x)), __dmul_rn(2.0, d.fa));
+    double pref = 3.0 / (2.0 * x2 * x2 * cubic);
     return d.flux_scale * pref * br;
 }
 
@@ -458,14 +462,14 @@ __device__ __forceinline__ double redshift64(const ImageDesc& d, double r, doubl
         double M = d.M, a = d.a;
         g[0] = -(1.0 - 2.0 * M / r);
         g[1] = -2.0 * M * a / r;
-        g[4] = r * r + a * a + 2.0 * M * a * a / r;
+        g[4] = __dadd_rn(__dadd_rn(__dmul_rn(r, r), __dmul_rn(a, a)), 2.0 * M * a * a / r);
     } else {
         lower64<METRIC>(d, r, kHalfPi, g);
     }
-    double Om = d.sqrtM / (r * sqrt(r) + d.a * d.sqrtM);
-    double ut = 1.0 / sqrt(-g[0] - 2.0 * Om * g[1] - Om * Om * g[4]);
+    double Om = d.sqrtM / __dadd_rn(__dmul_rn(r, sqrt(r)), __dmul_rn(d.a, d.sqrtM));
+    double ut = 1.0 / sqrt(__dsub_rn(__dsub_rn(-g[0], __dmul_rn(2.0 * Om, g[1])), __dmul_rn(__dmul_rn(Om, Om), g[4])));
     if (!d.doppler) return 1.0 / ut;
-    return pt / (ut * (pt + Om * pph));
+    return pt / (ut * __dadd_rn(pt, __dmul_rn(Om, pph)));
 }
 
 // ---------------------------------------------------------------------------

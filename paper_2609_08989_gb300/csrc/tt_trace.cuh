@@ -637,21 +637,49 @@ static __device__ float initial_step32(const Ray32& f32, const StateF& f0, const
     return fminf(100.0f * h0, h1);
 }
 
-// An image (or a pixel range of whole rows) whose width is a multiple of 8 and
-// whose row count is a multiple of 4 is handed out in 8 x 4 pixel tiles (32
-// consecutive queue entries per tile), so that the rays a warp takes together
-// start close on the sky and stay in step: the queue entry q of such a range
-// traces the tile's pixel returned here (relative to the range's first pixel).
-// Outputs are per pixel either way.
+// The k-th of n places ordered outward from place c: c, c + 1, c - 1, c + 2, ...,
+// and what is left of the longer side.
+__device__ __forceinline__ long long outward(long long k, long long n, long long c) {
+    const long long below = c, above = n - 1 - c, m = min(below, above);
+    if (k <= 2 * m) return (k & 1) ? c + ((k + 1) >> 1) : c - (k >> 1);
+    return above > below ? c + (k - m) : c - (k - m);
+}
+
+// The pixel (relative to the range's first) that queue entry q of an image or a
+// pixel range traces; outputs are per pixel either way.
+//
+// A range of whole rows whose width is a multiple of 8 and whose row count is a
+// multiple of 4 is handed out in 8 x 4 pixel tiles (32 consecutive queue entries
+// per tile), so that the rays a warp takes together start close on the sky and
+// stay in step; others in runs of 32 pixels.
+//
+// OUTWARD: tile rows (or runs) are taken outward from the line beta = 0.  The
+// longest rays, those that circle the hole, pass near it, at most ~7 M away;
+// taken in order of beta they start when half of the image is done, and with few
+// rays per lane the last of them run on a GPU that is otherwise empty: the
+// double-float table image of 512^2 (6.7 rays per lane) 310 -> 268 ms, of 768^2
+// 560 -> 491 ms; FP64 384^2 32.3 -> 29.0 ms, double-float 256^2 6.4 -> 5.3 ms, the
+// prescribed split's 1024^2 35.1 -> 32.2 ms; no change with one ray per lane or
+// with many.  The mixed kernels whose near-critical rays run apart have no such
+// tail, and are 2-10 % slower when the rays that need zone steps come all at
+// once (768^2 8.8 -> 9.8 ms, 2048^2 38.1 -> 39.1 ms): they keep the order of beta.
+template <bool OUTWARD>
 __device__ __forceinline__ long long tile_pixel(const ImageDesc& d, long long q) {
     const long long band = 4LL * d.nx;
+    // the row of beta = 0, within the range (an undefined quotient gives some row)
+    const double j0 = fmin(fmax(-d.beta_min / d.dbeta, 0.0), 2147483647.0);
+    const long long mid = (long long)j0 * d.nx + d.nx / 2 - d.pix_begin;
     if ((d.nx & 7) == 0 && d.pix_begin % band == 0 && d.pix_count % band == 0) {
-        const long long tile = q >> 5, tiles_x = d.nx >> 3;
-        const long long ty = tile / tiles_x, tx = tile - ty * tiles_x;
+        const long long tile = q >> 5, tiles_x = d.nx >> 3, rows = d.pix_count / band;
+        long long ty = tile / tiles_x;
+        const long long tx = tile - ty * tiles_x;
         const int lane = (int)(q & 31);
-        q = (ty * 4 + (lane >> 3)) * d.nx + tx * 8 + (lane & 7);
+        if (OUTWARD) ty = outward(ty, rows, min(max(mid / band, 0LL), rows - 1));
+        return (ty * 4 + (lane >> 3)) * d.nx + tx * 8 + (lane & 7);
     }
-    return q;
+    const long long runs = d.pix_count >> 5, run = q >> 5;     // (a last part of a run keeps its place)
+    if (!OUTWARD || run >= runs) return q;
+    return outward(run, runs, min(max(mid >> 5, 0LL), runs - 1)) * 32 + (q & 31);
 }
 
 // ---------------------------------------------------------------------------
@@ -832,7 +860,7 @@ __device__ __forceinline__ void record_crossing(Lane& L, double rc, const Solver
             TT_STORE(d, r_cross, L.nrec * n + q, kMaxCross * n, rc);
             TT_STORE(d, g, L.nrec * n + q, kMaxCross * n, gf);
             TT_STORE(d, I_cross, L.nrec * n + q, kMaxCross * n, I);
-            L.cold().inten += I;
+            L.cold().inten = __dadd_rn(L.cold().inten, I);
             L.nrec++;
         }
         L.ncross++;
@@ -1524,6 +1552,7 @@ __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, l
     static_assert(PREC == 0 || METHOD == 0, "the mixed and double-float paths step with Dormand-Prince");
     constexpr int ACC = (PREC == 2 || PREC == 3) ? 1 : 0;
     constexpr bool MIX = (PREC == 1 || PREC == 2 || PREC == 4);
+    constexpr bool OUTWARD = !(PREC == 1 || PREC == 2);
     if constexpr (PREC != 0) {
         df_sincos_table(s_df_tab);
         if constexpr (METRIC == 1) df_log_table(s_df_ln);
@@ -1556,7 +1585,7 @@ __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, l
                     if (rid < total) {
                         const int im = (n_desc == 1) ? 0 : find_image(descs, n_desc, rid);
                         const ImageDesc* dp = descs + im;
-                        const long long q = tile_pixel(*dp, rid - dp->ray_begin);
+                        const long long q = tile_pixel<OUTWARD>(*dp, rid - dp->ray_begin);
                         const bool skip = MIX && band > 0.0f && near_critical(*dp, q, band);
                         if (!skip && init_ray<METRIC>(L, dp, q, sol)) {
                             st = kRun;
@@ -1704,7 +1733,7 @@ __device__ __forceinline__ void critical_loop(const ImageDesc* descs, int n_desc
                     if (rid < total) {
                         const int im = (n_desc == 1) ? 0 : find_image(descs, n_desc, rid);
                         const ImageDesc* dp = descs + im;
-                        const long long q = tile_pixel(*dp, rid - dp->ray_begin);
+                        const long long q = tile_pixel<false>(*dp, rid - dp->ray_begin);
                         if (near_critical(*dp, q, band) && init_ray<0>(L, dp, q, solc, true)) {
                             st = kRun;
                             if (ACC == 1) split_state(L.y, yhi, L.lo);
