@@ -74,14 +74,45 @@ __device__ __forceinline__ void flow64_near(const ImageDesc& d, const KerrK& kk,
 
 // Products with the flow k1, the coefficients h a_ij and (s0, c0) are formed by
 // m: for IntMul, k1, h, s0 and c0 are checked here, k2 .. k6 in their flows.
+//
+// A rolled loop: the sums over earlier stages are kept per later stage (S3 .. S7
+// and the error estimate) and each new flow is added to those that take it, in
+// the order of the stages, so that one copy of the flow serves all of them.
+// Stages 2-4 take coefficients pre-multiplied by h (one multiply each, shared by
+// the four components), their sums starting from y.
+template <class T>
+struct RkWeights {          // of the flow of stage j + 2: a_5j, a_6j, b_j, e_j
+    double w[5][4] = {{T::a52, T::a62, 0.0, 0.0},
+                      {T::a53, T::a63, T::b3, T::e3},
+                      {T::a54, T::a64, T::b4, T::e4},
+                      {0.0, T::a65, T::b5, T::e5},
+                      {0.0, 0.0, T::b6, T::e6}};
+};
+
+template <class T>
+static __constant__ RkWeights<T> kRkWeights = {};
+
+__device__ __forceinline__ void add_to(State& s, double w, const State& k) {
+    s = State{fma(w, k.r, s.r), fma(w, k.th, s.th), fma(w, k.pr, s.pr), fma(w, k.pth, s.pth)};
+}
+
+__device__ __forceinline__ State plus(const State& y, double h, const State& k) {
+    return State{fma(h, k.r, y.r), fma(h, k.th, y.th), fma(h, k.pr, y.pr), fma(h, k.pth, y.pth)};
+}
+
+template <class Mul>
+__device__ __forceinline__ State times(const State& k, double w, Mul& m) {
+    return State{m.mul(k.r, w), m.mul(k.th, w), m.mul(k.pr, w), m.mul(k.pth, w)};
+}
+
 template <int METRIC, int METHOD, class Mul>
 __device__ __forceinline__ void rk_step64(const ImageDesc& d, const KerrK& kk, const RayConst& R,
                                            const State& y, const State& k1, double h, State& yn,
                                            State& kn, double& Hn, State& err, double s0, double c0,
                                            double& sn, double& cn, Mul& m) {
     using T = RK<METHOD>;
-    State k2, k3, k4, k5, k6, ys;
-    double Hs, ss = s0, cs = c0;
+    sn = s0;
+    cn = c0;
     m.see(h);
     m.see(k1.r);
     m.see(k1.th);
@@ -91,56 +122,39 @@ __device__ __forceinline__ void rk_step64(const ImageDesc& d, const KerrK& kk, c
         m.see(s0);
         m.see(c0);
     }
-#define TT_STAGE(dst, expr_r, expr_t, expr_p, expr_q)                                \
-    ys.r = fma(h, (expr_r), y.r);                                                    \
-    ys.th = fma(h, (expr_t), y.th);                                                  \
-    ys.pr = fma(h, (expr_p), y.pr);                                                  \
-    ys.pth = fma(h, (expr_q), y.pth);                                                \
-    flow64_near<METRIC>(d, kk, R, ys, y.th, s0, c0, dst, Hs, ss, cs, m);
-// stages 2-4: coefficients pre-multiplied by h (one multiply each, shared by
-// the four components), the stage point an FMA chain from y
-#define TT_PSTAGE(dst, EXPR)                                                         \
-    ys.r = EXPR(r);                                                                  \
-    ys.th = EXPR(th);                                                                \
-    ys.pr = EXPR(pr);                                                                \
-    ys.pth = EXPR(pth);                                                              \
-    flow64_near<METRIC>(d, kk, R, ys, y.th, s0, c0, dst, Hs, ss, cs, m);
-    const double h21 = m.mul(h, T::a21), h31 = m.mul(h, T::a31), h32 = m.mul(h, T::a32);
-    const double h41 = m.mul(h, T::a41), h42 = m.mul(h, T::a42), h43 = m.mul(h, T::a43);
-#define TT_P2(f) fma(h21, k1.f, y.f)
-#define TT_P3(f) fma(h32, k2.f, fma(h31, k1.f, y.f))
-#define TT_P4(f) fma(h43, k3.f, fma(h42, k2.f, fma(h41, k1.f, y.f)))
-#define TT_C5(f) fma(T::a54, k4.f, fma(T::a53, k3.f, fma(T::a52, k2.f, m.mul(k1.f, T::a51))))
-#define TT_C6(f) fma(T::a65, k5.f, fma(T::a64, k4.f, fma(T::a63, k3.f, fma(T::a62, k2.f, m.mul(k1.f, T::a61)))))
-#define TT_C7(f) fma(T::b6, k6.f, TT_MAC(T::b5, k5.f, fma(T::b4, k4.f, fma(T::b3, k3.f, m.mul(k1.f, T::b1)))))
-    TT_PSTAGE(k2, TT_P2)
-    TT_PSTAGE(k3, TT_P3)
-    TT_PSTAGE(k4, TT_P4)
-    TT_STAGE(k5, TT_C5(r), TT_C5(th), TT_C5(pr), TT_C5(pth))
-    TT_STAGE(k6, TT_C6(r), TT_C6(th), TT_C6(pr), TT_C6(pth))
-    yn.r = fma(h, TT_C7(r), y.r);
-    yn.th = fma(h, TT_C7(th), y.th);
-    yn.pr = fma(h, TT_C7(pr), y.pr);
-    yn.pth = fma(h, TT_C7(pth), y.pth);
-    flow64_near<METRIC>(d, kk, R, yn, y.th, s0, c0, kn, Hn, ss, cs, m);
-    sn = ss;
-    cn = cs;
-// the error vector without its factor h (err_norm2 applies it once)
-#define TT_E(f) \
-    TT_MAC(T::e7, kn.f, fma(T::e6, k6.f, fma(T::e5, k5.f, fma(T::e4, k4.f, fma(T::e3, k3.f, m.mul(k1.f, T::e1))))))
-    err.r = TT_E(r);
-    err.th = TT_E(th);
-    err.pr = TT_E(pr);
-    err.pth = TT_E(pth);
-#undef TT_E
-#undef TT_STAGE
-#undef TT_PSTAGE
-#undef TT_P2
-#undef TT_P3
-#undef TT_P4
-#undef TT_C5
-#undef TT_C6
-#undef TT_C7
+    const double h32 = m.mul(h, T::a32), h42 = m.mul(h, T::a42), h43 = m.mul(h, T::a43);
+    State ys = plus(y, m.mul(h, T::a21), k1);
+    State S3 = plus(y, m.mul(h, T::a31), k1), S4 = plus(y, m.mul(h, T::a41), k1);
+    State S5 = times(k1, T::a51, m), S6 = times(k1, T::a61, m), S7 = times(k1, T::b1, m);
+    err = times(k1, T::e1, m);          // the error vector without its factor h (err_norm2 applies it once)
+#pragma unroll 1
+    for (int j = 2;; ++j) {
+        State k;
+        flow64_near<METRIC>(d, kk, R, ys, y.th, s0, c0, k, Hn, sn, cn, m);
+        if (j == 7) {
+            kn = k;
+            break;
+        }
+        const double* w = kRkWeights<T>.w[j - 2];
+        if (j <= 4) add_to(S5, w[0], k);
+        if (j <= 5) add_to(S6, w[1], k);
+        if (j >= 3) {
+            if (w[2] != 0.0) add_to(S7, w[2], k);
+            add_to(err, w[3], k);
+        }
+        if (j == 2) {
+            add_to(S3, h32, k);
+            add_to(S4, h42, k);
+            ys = S3;
+        } else if (j == 3) {
+            add_to(S4, h43, k);
+            ys = S4;
+        } else {
+            ys = plus(y, h, j == 4 ? S5 : j == 5 ? S6 : S7);
+        }
+    }
+    yn = ys;
+    if (T::e7 != 0.0) add_to(err, T::e7, kn);
 }
 
 // ---------------------------------------------------------------------------
