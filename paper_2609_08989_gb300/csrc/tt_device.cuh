@@ -105,8 +105,7 @@ struct State {
 // formed by m (tt_soft64.cuh).  For IntMul the checks leave every product that
 // is not checked itself with two factors that are normal: r, p_r, s, c and SD
 // lie in 2^+-100, so Sigma, Delta, 1/Sigma, 1/Delta and 1/sin^2 lie in 2^+-300.
-// K cancels to ~1e-16 of its terms, at times to zero: its product with 1/Sigma
-// is always a plain one.
+// K cancels to ~1e-16 of its terms, at times to zero.
 template <class Mul>
 __device__ __forceinline__ void kerr_flow64_sc(const KerrK& k, const RayConst& R, const State& y, double s,
                                                double c, State& f, double& H, Mul& m) {
@@ -133,7 +132,7 @@ __device__ __forceinline__ void kerr_flow64_sc(const KerrK& k, const RayConst& R
     K = fma(y.pth, y.pth, K);
     K = fma(Del, pr2, K);
     K = fma(-A, AiD, K);
-    const double H2 = K * iS;
+    const double H2 = m.mulz(K, iS);
     H = 0.5 * H2;
     const double q1 = fma(R.pt2, AiD, H2);
     const double q2 = fma(AiD, AiD, pr2);
@@ -141,8 +140,8 @@ __device__ __forceinline__ void kerr_flow64_sc(const KerrK& k, const RayConst& R
     const double t2 = fma(k.a2, H2, t1);
     f.r = m.mul(m.mul(Del, y.pr), iS);
     f.th = m.chk(y.pth, iS);
-    f.pr = m.chk(fma(r, q1, -m.chk(r - k.M, q2)), iS);
-    f.pth = m.chk(-m.mul(sc, iS), t2);
+    f.pr = m.chk(fma(r, q1, m.neg(m.chk(r - k.M, q2))), iS);
+    f.pth = m.chk(m.neg(m.mul(sc, iS)), t2);
 }
 
 __device__ __forceinline__ void kerr_flow64(const KerrK& k, const RayConst& R, const State& y, State& f,
@@ -164,19 +163,35 @@ template <class Mul>
 __device__ __forceinline__ void sincos_near(double th, double th0, double s0, double c0, double& s, double& c,
                                             Mul& m) {
     const double d = th - th0;
-    if (abs_below_hi(d, kHi0p01)) {
+    if (Mul::kInt && abs_below_hi(d, kHi0p01)) {
+        // the series below in significands: every term is smaller than its
+        // constant and of the other sign, so each sum stays in a binade that is
+        // known (the LSB of 1/6 - .. is 2^-55, of 1/24 - .. 2^-57, of 1/2 - .. 2^-54,
+        // of 1 - .. 2^-53), and no sign or normalisation is left to work out
+        const double d2 = m.mul(d, d);
+        const Sig53 x = sig53(d2);
+        const unsigned e = (unsigned)__double2hiint(d2) >> 20;
+        const Sig53 p1 = soft_sub_from(frame64(1.0 / 6.0), sig53(1.0 / 120.0), x, 1027u - e);
+        const Sig53 p2 = soft_sub_from(1ull << 63, p1, x, 1025u - e);
+        const Sig53 q1 = soft_sub_from(frame64(1.0 / 24.0), sig53(1.0 / 720.0), x, 1028u - e);
+        const Sig53 q2 = soft_sub_from(1ull << 63, q1, x, 1026u - e);
+        const Sig53 q3 = soft_sub_from(1ull << 63, q2, x, 1024u - e);
+        const double sd = m.chk(d, near_one(p2)), cd = near_one(q3);
+        s = fma(s0, cd, m.mul(c0, sd));
+        c = fma(c0, cd, m.neg(m.mul(s0, sd)));
+    } else if (abs_below_hi(d, kHi0p01)) {
         const double d2 = m.mul(d, d);
         const double sd = m.chk(d, fma(d2, fma(d2, 1.0 / 120.0, -1.0 / 6.0), 1.0));
         const double cd = fma(d2, fma(d2, fma(d2, -1.0 / 720.0, 1.0 / 24.0), -0.5), 1.0);
         s = fma(s0, cd, m.mul(c0, sd));
-        c = fma(c0, cd, -m.mul(s0, sd));
+        c = fma(c0, cd, m.neg(m.mul(s0, sd)));
     } else if (abs_below_hi(d, kHi0p1)) {
         const double d2 = m.mul(d, d);
         const double sd = m.chk(
             d, fma(d2, fma(d2, fma(d2, fma(d2, 1.0 / 362880.0, -1.0 / 5040.0), 1.0 / 120.0), -1.0 / 6.0), 1.0));
         const double cd = fma(d2, fma(d2, fma(d2, fma(d2, 1.0 / 40320.0, -1.0 / 720.0), 1.0 / 24.0), -0.5), 1.0);
         s = fma(s0, cd, m.mul(c0, sd));
-        c = fma(c0, cd, -m.mul(s0, sd));
+        c = fma(c0, cd, m.neg(m.mul(s0, sd)));
     } else {
         sincos(th, &s, &c);
     }

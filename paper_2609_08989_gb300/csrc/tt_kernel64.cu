@@ -22,8 +22,8 @@ __global__ void __launch_bounds__(384) trace_kernel64_b384(const __grid_constant
 // Register-capped builds of the closed-form Kerr kernel (128 threads): at least
 // MINB resident blocks per SM caps registers at 65536 / (128 MINB) per thread
 // (MINB 3: 168, MINB 4: 128).
-template <int MINB>
-__global__ void __launch_bounds__(128, MINB) trace_kernel64_regcap(const __grid_constant__ LaunchParams<1> p) {
+template <int MINB, int N>
+__global__ void __launch_bounds__(128, MINB) trace_kernel64_regcap(const __grid_constant__ LaunchParams<N> p) {
     trace_loop<0, 0>(p.desc, p.n_desc, p.total, p.sol, p.tune, p.queue);
 }
 
@@ -51,10 +51,16 @@ static cudaError_t launch64(const ImageDesc* descs, int n, long long total, int 
         if (shape.block == 256) return launch_persistent<N>(trace_kernel64_b256<0, N>, 256, bps, p, stream);
         if (shape.block == 384) return launch_persistent<N>(trace_kernel64_b384<0, N>, 384, bps, p, stream);
         if constexpr (N == 1) {
-            if (shape.reg_variant == 1) return launch_persistent<N>(trace_kernel64_regcap<3>, 128, bps, p, stream);
-            if (shape.reg_variant == 2) return launch_persistent<N>(trace_kernel64_regcap<4>, 128, bps, p, stream);
+            if (shape.reg_variant == 2) return launch_persistent<N>(trace_kernel64_regcap<4, N>, 128, bps, p, stream);
+            // the uncapped build (206 registers, two blocks per SM, no spills) where
+            // every ray has a lane of its own, so that the longest ray sets the time
+            // (64^2 shadow 11.9 ms, capped 13.3); else three blocks per SM (1024^2 disk
+            // 152.1 ms, uncapped 157.7): the FP64 unit then waits less for warps that
+            // are in their integer products
+            const bool few = total <= 2LL * 128 * sm_count();
+            if (shape.reg_variant == 0 && few) return launch_persistent<N>(trace_kernel64<0, N>, 128, bps, p, stream);
         }
-        return launch_persistent<N>(trace_kernel64<0, N>, 128, bps, p, stream);
+        return launch_persistent<N>(trace_kernel64_regcap<3, N>, 128, bps, p, stream);
     }
     if (metric_mode == 1) return launch_persistent<N>(trace_kernel64<1, N>, 128, bps, p, stream);
     return cudaErrorInvalidValue;

@@ -10,8 +10,8 @@
 
 namespace tt {
 
-template <int METHOD, int METRIC, int N, int BLOCK>
-__global__ void __launch_bounds__(BLOCK) trace_kernel_rk(const __grid_constant__ LaunchParams<N> p) {
+template <int METHOD, int METRIC, int N, int BLOCK, int MINB = 1>
+__global__ void __launch_bounds__(BLOCK, MINB) trace_kernel_rk(const __grid_constant__ LaunchParams<N> p) {
     trace_loop<METRIC, 0, METHOD>(p.desc, p.n_desc, p.total, p.sol, p.tune, p.queue);
 }
 
@@ -24,6 +24,12 @@ static cudaError_t launch_rk_n(const ImageDesc* descs, int n, long long total, i
     const int bps = shape.blocks_per_sm;
     if (metric_mode == 0) {
         if (shape.block >= 256) return launch_persistent<N>(trace_kernel_rk<METHOD, 0, N, 256>, 256, bps, p, stream);
+        // the pairs, as Dormand-Prince: three blocks per SM unless every ray has a
+        // lane of its own
+        if constexpr (METHOD <= 2) {
+            if (total > 2LL * 128 * sm_count())
+                return launch_persistent<N>(trace_kernel_rk<METHOD, 0, N, 128, 3>, 128, bps, p, stream);
+        }
         return launch_persistent<N>(trace_kernel_rk<METHOD, 0, N, 128>, 128, bps, p, stream);
     }
     if (metric_mode == 1) return launch_persistent<N>(trace_kernel_rk<METHOD, 1, N, 128>, 128, bps, p, stream);

@@ -51,6 +51,62 @@ __device__ __forceinline__ double soft_mul64(double a, double b) {
     return __hiloint2double((int)hi, (int)lo);
 }
 
+// The significand of a normal double as an integer in [2^52, 2^53) (2^53 for a
+// result rounded up to the next binade).
+struct Sig53 {
+    unsigned m, l;          // the high 21 (22) and the low 32 bits
+};
+
+__device__ __forceinline__ Sig53 sig53(double x) {
+    return Sig53{((unsigned)__double2hiint(x) & 0xfffffu) | 0x100000u, (unsigned)__double2loint(x)};
+}
+
+// |x| in units of its LSB / 2^10
+__device__ __forceinline__ unsigned long long frame64(double x) {
+    const Sig53 a = sig53(x);
+    return (((unsigned long long)a.m << 32) | a.l) << 10;
+}
+
+// the double a 2^-53, a in [2^52, 2^53]
+__device__ __forceinline__ double near_one(Sig53 a) {
+    return __hiloint2double((int)(a.m - 0x100000u + (1022u << 20)), (int)a.l);
+}
+
+// |c| - |a b|, rounded to nearest even, for |a b| < |c| / 16 and a result whose
+// LSB L is known: its significand.  c64 = |c| / (L / 2^10); the product's upper 64
+// bits, P = a b / 2^42, are 2^n times that unit.  ~26 integer instructions: 12
+// cycles per warp and SM against 16 of the FP64 unit.
+__device__ __forceinline__ Sig53 soft_sub_from(unsigned long long c64, Sig53 a, Sig53 b, unsigned n) {
+    typedef unsigned long long u64;
+    const u64 w0 = (u64)a.l * b.l;
+    const u64 w1 = (u64)a.m * b.l + (w0 >> 32);
+    const u64 w2 = (u64)a.l * b.m + w1;
+    const u64 w3 = (u64)a.m * b.m + (w2 >> 32);
+    const unsigned z = (unsigned)w2, t = (unsigned)w0;
+    // the product's upper 64 bits, in units of 2^n of the result's frame
+    const u64 p = (w3 << 22) | (z >> 10);
+    const unsigned rest = (z << 22) | t;
+    u64 q, back;            // (these shifts give 0 for n >= 64)
+    asm("shr.u64 %0, %1, %2;" : "=l"(q) : "l"(p), "r"(n));
+    asm("shl.b64 %0, %1, %2;" : "=l"(back) : "l"(q), "r"(n));
+    const u64 lost = back ^ p;
+    const unsigned sticky = min((unsigned)lost | (unsigned)(lost >> 32) | rest, 1u);
+    const u64 r = c64 - q - sticky;
+    const unsigned rl = (unsigned)r, rh = (unsigned)(r >> 32);
+    const unsigned ml = __funnelshift_r(rl, rh, 10), mh = rh >> 10;
+    const unsigned up = ((ml & 1u) | sticky) + 0x7fffffffu;
+    Sig53 o;
+    asm("{\n\t"
+        ".reg .u32 d;\n\t"
+        "add.cc.u32 d, %2, %3;\n\t"
+        "addc.cc.u32 %0, %4, 0;\n\t"
+        "addc.u32 %1, %5, 0;\n\t"
+        "}"
+        : "=r"(o.l), "=r"(o.m)
+        : "r"(rl << 22), "r"(up), "r"(ml), "r"(mh));
+    return o;
+}
+
 // How a block of FP64 arithmetic forms its products.
 //   mul(a, b)  the product
 //   chk(a, b)  the product, whose magnitude is to lie in 2^-100 .. 2^100
@@ -62,14 +118,40 @@ __device__ __forceinline__ double soft_mul64(double a, double b) {
 // bit either way.  A checked product is reliable when one factor is known to be
 // normal and within 2^+-700: the exponent field of a product with a zero,
 // subnormal, infinite or NaN factor then falls outside the window.
+//   neg(x)     -x
+//   mulz(a, b) the product where a may be zero
+//   chkw(a, b) the same, whose magnitude is to be zero or in 2^-400 .. 2^400
 struct FpMul {
+    static constexpr bool kInt = false;
+    __device__ __forceinline__ double neg(double x) { return -x; }
+    __device__ __forceinline__ double mulz(double a, double b) { return a * b; }
+    __device__ __forceinline__ double chkw(double a, double b) { return a * b; }
     __device__ __forceinline__ double mul(double a, double b) { return a * b; }
     __device__ __forceinline__ double chk(double a, double b) { return a * b; }
     __device__ __forceinline__ void see(double) {}
 };
 
 struct IntMul {
+    static constexpr bool kInt = true;
+    // (the sign bit of a product that integer instructions made: as a floating-point
+    // negation it was a DADD)
+    __device__ __forceinline__ double neg(double x) {
+        return __hiloint2double(__double2hiint(x) ^ 0x80000000, __double2loint(x));
+    }
     unsigned bad = 0;
+    __device__ __forceinline__ double mulz(double a, double b) {
+        const bool zero = ((__double2hiint(a) << 1) | __double2loint(a)) == 0;
+        const double p = soft_mul64(a, b);
+        see(zero ? 1.0 : p);
+        return zero ? __hiloint2double((__double2hiint(a) ^ __double2hiint(b)) & 0x80000000, 0) : p;
+    }
+    __device__ __forceinline__ double chkw(double a, double b) {
+        const bool zero = ((__double2hiint(a) << 1) | __double2loint(a)) == 0;
+        const double p = soft_mul64(a, b);
+        const unsigned hi = zero ? 1023u << 20 : (unsigned)__double2hiint(p);
+        bad = max(bad, (hi + hi - ((1023u - 400u) << 21)) >> 2);
+        return zero ? __hiloint2double((__double2hiint(a) ^ __double2hiint(b)) & 0x80000000, 0) : p;
+    }
     __device__ __forceinline__ double mul(double a, double b) { return soft_mul64(a, b); }
     __device__ __forceinline__ double chk(double a, double b) {
         const double p = soft_mul64(a, b);

@@ -39,15 +39,28 @@ constexpr unsigned kFull = 0xffffffffu;
 // x^(-1/10) for the step-size factor: the SFU's single-precision power refined
 // by one Newton step of y^-10 = x, y <- y (1.1 - 0.1 x y^10), which squares the
 // relative error (~1e-7 -> ~1e-13).  Callers handle x < 1e-30 themselves.
-__device__ __forceinline__ double pow_m01(double x) {
+template <class Mul>
+__device__ __forceinline__ double pow_m01(double x, Mul& m) {
     double y = (double)__powf((float)x, -0.1f);
-    double y2 = y * y, y4 = y2 * y2, y10 = y4 * y4 * y2;
-    return y * fma(-0.1 * x, y10, 1.1);
+    double y2 = m.mul(y, y), y4 = m.mul(y2, y2), y10 = m.mul(m.mul(y4, y4), y2);
+    return m.mul(y, fma(m.mul(-0.1, x), y10, 1.1));
 }
 
 // Step-size factor 0.9 err^(-1/5) from err^2 (large when err^2 is tiny or 0).
 __device__ __forceinline__ double step_factor(double err2) {
-    return lt_pos(err2, 1e-30) ? 1e30 : 0.9 * pow_m01(err2);
+    FpMul m;
+    return lt_pos(err2, 1e-30) ? 1e30 : 0.9 * pow_m01(err2, m);
+}
+
+// h min(top, max(0.2, step_factor(err2))) for 0 < h <= 2^100: on the integer
+// pipes where err2 is at most 2^100 (the factor is then finite and positive).
+__device__ __forceinline__ double next_h(double h, double err2, double top) {
+    if (!lt_pos(err2, 0x1p100)) return h * fmin(top, fmax(0.2, step_factor(err2)));
+    IntMul m;
+    double f = lt_pos(err2, 1e-30) ? 1e30 : m.mul(0.9, pow_m01(err2, m));
+    f = lt_pos(f, 0.2) ? 0.2 : f;
+    f = lt_pos(top, f) ? top : f;
+    return m.mul(h, f);
 }
 
 // ---------------------------------------------------------------------------
@@ -143,12 +156,10 @@ __device__ __forceinline__ void rk_step64(const ImageDesc& d, const KerrK& kk, c
             add_to(err, w[3], k);
         }
         if (j == 2) {
-            add_to(S3, h32, k);
-            add_to(S4, h42, k);
-            ys = S3;
+            ys = plus(S3, h32, k);
+            S4 = plus(S4, h42, k);
         } else if (j == 3) {
-            add_to(S4, h43, k);
-            ys = S4;
+            ys = plus(S4, h43, k);
         } else {
             ys = plus(y, h, j == 4 ? S5 : j == 5 ? S6 : S7);
         }
@@ -336,9 +347,9 @@ __device__ __forceinline__ double err_norm2(const State& y, const State& yn, con
     asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(inv) : "d"(pp));
     inv = m.mul(fma(inv, fma(-pp, inv, 1.0), inv), he);
     const double i01 = m.mul(inv, p23), i23 = m.mul(inv, p01);   // he/(s0 s1), he/(s2 s3)
-    const double q0 = (e.r * s1) * i01, q1 = (e.th * s0) * i01;
-    const double q2 = (e.pr * s3) * i23, q3 = (e.pth * s2) * i23;
-    return 0.25 * fma(q3, q3, fma(q2, q2, fma(q1, q1, q0 * q0)));
+    const double q0 = m.chkw(m.chkw(e.r, s1), i01), q1 = m.chkw(m.chkw(e.th, s0), i01);
+    const double q2 = m.chkw(m.chkw(e.pr, s3), i23), q3 = m.chkw(m.chkw(e.pth, s2), i23);
+    return 0.25 * fma(q3, q3, fma(q2, q2, fma(q1, q1, m.chkw(q0, q0))));
 }
 
 // Non-finite tests on the exponent bits (integer pipe, not the FP64 pipe).
@@ -1028,6 +1039,7 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
     if (lt_pos(L.h, hmin)) return 3;
     State yn, kn, e;
     double Hn, sn = L.s0, cn = L.c0, err2;
+    bool fast = false;                         // the attempt's products were integer ones
     if constexpr (METHOD == 4) {
         verlet_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn);
         err2 = 0.0;                            // fixed step, always accepted
@@ -1044,7 +1056,8 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
         IntMul m;
         rk_step64<METRIC, METHOD>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
         err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
-        if (!(m.ok() && sol.int_mul)) {
+        fast = m.ok() && sol.int_mul;
+        if (!fast) {
             const Step64 o = plain_step64<METHOD>(&d, L.kk, L.cold().R, L.y, L.k1, L.h, L.s0, L.c0, sol.atol, sol.rtol);
             yn = o.yn;
             kn = o.kn;
@@ -1083,7 +1096,9 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
         if constexpr (METHOD == 3) {
             L.h *= fmin(L.last_rej ? 1.0 : 4.0, fmax(0.02, gbs_factor(err2)));
         } else if constexpr (METHOD != 4) {
-            L.h *= fmin(L.last_rej ? 1.0 : 10.0, fmax(0.2, step_factor(err2)));
+            const double top = L.last_rej ? 1.0 : 10.0;
+            if (fast) L.h = next_h(L.h, err2, top);
+            else L.h *= fmin(top, fmax(0.2, step_factor(err2)));
         }
         L.last_rej = false;
     } else {
@@ -1091,7 +1106,8 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
         if constexpr (METHOD == 3) {
             L.h *= fmin(1.0, fmax(0.02, gbs_factor(err2)));
         } else {
-            L.h *= fmax(0.2, step_factor(err2));
+            if (fast) L.h = next_h(L.h, err2, 1.0);
+            else L.h *= fmax(0.2, step_factor(err2));
         }
         L.last_rej = true;
     }
