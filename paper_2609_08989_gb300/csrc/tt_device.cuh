@@ -26,6 +26,7 @@ __device__ __forceinline__ bool le_pos(double x, double y) { return __double_as_
 // |x| below a threshold given by the high 32 bits of a positive double.
 __device__ __forceinline__ bool abs_below_hi(double x, int hi) { return (__double2hiint(x) & 0x7fffffff) < hi; }
 constexpr int kHi0p01 = 0x3F847AE1;    // high word of 0.01 (the threshold is 0.01 - 3e-11)
+constexpr int kHi1e5 = 0x40F86A00;     // high word of 1e5
 constexpr int kHi0p1 = 0x3FB99999;     // high word of 0.1 (the threshold is 0.1 - 4e-10)
 
 // ---------------------------------------------------------------------------

@@ -111,6 +111,7 @@ __device__ __forceinline__ Sig53 soft_sub_from(unsigned long long c64, Sig53 a, 
 //   mul(a, b)  the product
 //   chk(a, b)  the product, whose magnitude is to lie in 2^-100 .. 2^100
 //   see(x)     x, which is to lie there
+//   must(b)    b is to hold
 // With FpMul all three are plain FP64.  With IntMul products are formed on the
 // integer pipes and `bad` collects what lies outside (zeros, infinities, NaNs,
 // subnormals included): when ok() is false at the end the block's results are
@@ -129,6 +130,7 @@ struct FpMul {
     __device__ __forceinline__ double mul(double a, double b) { return a * b; }
     __device__ __forceinline__ double chk(double a, double b) { return a * b; }
     __device__ __forceinline__ void see(double) {}
+    __device__ __forceinline__ void must(bool) {}
 };
 
 struct IntMul {
@@ -163,6 +165,7 @@ struct IntMul {
         const unsigned hi = (unsigned)__double2hiint(x);
         bad = max(bad, hi + hi - ((1023u - 100u) << 21));
     }
+    __device__ __forceinline__ void must(bool b) { bad = b ? bad : ~0u; }
     __device__ __forceinline__ bool ok() const { return bad < (200u << 21); }
 };
 

@@ -175,8 +175,7 @@ __device__ __forceinline__ void rk_step64(const ImageDesc& d, const KerrK& kk, c
 // solution is the diagonal entry T_kk and the error T_kk - T_k,k-1.  Chain and
 // extrapolation run on the increment z - y (so the rounding in the error
 // estimate, a small difference of extrapolated values, scales with the step's
-// change rather than with |y|).  The table row lives in registers (the j and l
-// loops unroll, so each weight 1 / ((j / (j - l))^2 - 1) is a constant).
+// change rather than with |y|).  The table row lives in registers.
 // ---------------------------------------------------------------------------
 constexpr int kGbsK = 6;
 
@@ -192,16 +191,36 @@ __device__ __forceinline__ State add(const State& x, const State& y) {
     return State{x.r + y.r, x.th + y.th, x.pr + y.pr, x.pth + y.pth};
 }
 
+// Row J of the table: T[0] = d1 (T_J1), T[l] = T_J,l+1 from row J - 1.
+template <int J>
+__device__ __forceinline__ void gbs_row(State (&T)[kGbsK], const State& d1) {
+    State prev = T[0];                          // T_{J-1,1}
+    T[0] = d1;
+#pragma unroll
+    for (int l = 1; l < J; ++l) {
+        // 1 / ((J / (J - l))^2 - 1) as one quotient of integers
+        const double w = (double)((J - l) * (J - l)) / (double)(l * (2 * J - l));
+        const State old = T[l];                 // T_{J-1,l+1}
+        T[l] = axpy(w, sub(T[l - 1], prev), T[l - 1]);
+        prev = old;
+    }
+}
+
 // dT = T_kk - y, err = T_kk - T_k,k-1 for dz/dx = flow(z) from (y, f0 = flow(y)) over H.
+// One copy of the flow serves the sub-steps of every row (the six rows unrolled
+// with a flow each overflowed the instruction cache).
 template <class Flow>
 __device__ __forceinline__ void gbs_core(const State& y, const State& f0, double H, Flow&& flow, State& dT,
                                          State& err) {
     State T[kGbsK];
 #pragma unroll
+    for (int l = 0; l < kGbsK; ++l) T[l] = State{0.0, 0.0, 0.0, 0.0};
+#pragma unroll 1
     for (int j = 1; j <= kGbsK; ++j) {
         const double h = H / (double)(2 * j);
         State d0 = State{0.0, 0.0, 0.0, 0.0};
         State d1 = State{h * f0.r, h * f0.th, h * f0.pr, h * f0.pth};
+#pragma unroll 1
         for (int m = 1; m < 2 * j; ++m) {
             State fz;
             flow(add(y, d1), fz);
@@ -209,37 +228,48 @@ __device__ __forceinline__ void gbs_core(const State& y, const State& f0, double
             d0 = d1;
             d1 = d2;
         }
-        if (j == 1) {
-            T[0] = d1;
-        } else {
-            State prev = T[0];                  // T_{j-1,1}
-            T[0] = d1;
-#pragma unroll
-            for (int l = 1; l < j; ++l) {
-                // 1 / ((j / (j - l))^2 - 1) as one quotient of integers (rounded alike
-                // whether or not the loop unrolls into constants)
-                const double w = (double)((j - l) * (j - l)) / (double)(l * (2 * j - l));
-                const State old = T[l];         // T_{j-1,l+1}
-                T[l] = axpy(w, sub(T[l - 1], prev), T[l - 1]);
-                prev = old;
-            }
+        switch (j) {
+            case 1: gbs_row<1>(T, d1); break;
+            case 2: gbs_row<2>(T, d1); break;
+            case 3: gbs_row<3>(T, d1); break;
+            case 4: gbs_row<4>(T, d1); break;
+            case 5: gbs_row<5>(T, d1); break;
+            default: gbs_row<6>(T, d1); break;
         }
     }
     dT = T[kGbsK - 1];
     err = sub(T[kGbsK - 1], T[kGbsK - 2]);
 }
 
-template <int METRIC>
+// The flow with its products formed by m (closed-form metric; a table's are plain).
+template <int METRIC, class Mul>
+__device__ __forceinline__ void flow64_by(const ImageDesc& d, const KerrK& kk, const RayConst& R, const State& y,
+                                          State& f, double& H, Mul& m) {
+    if constexpr (METRIC == 0) {
+        double s, c;
+        if (Mul::kInt) {
+            // without sincos's branch for huge angles (they fail the check)
+            m.must(abs_below_hi(y.th, kHi1e5));
+            __builtin_assume(fabs(y.th) < 1e5);
+        }
+        sincos(y.th, &s, &c);
+        kerr_flow64_sc(kk, R, y, s, c, f, H, m);
+    } else {
+        flow64<METRIC>(d, kk, R, y, f, H);
+    }
+}
+
+template <int METRIC, class Mul>
 __device__ __forceinline__ void gbs_step64(const ImageDesc& d, const KerrK& kk, const RayConst& R,
                                            const State& y, const State& f0, double H, State& yn, State& kn,
-                                           double& Hn, State& err) {
+                                           double& Hn, State& err, Mul& m) {
     State dT;
     gbs_core(y, f0, H, [&](const State& z, State& fz) {
         double Hs;
-        flow64<METRIC>(d, kk, R, z, fz, Hs);
+        flow64_by<METRIC>(d, kk, R, z, fz, Hs, m);
     }, dT, err);
     yn = add(y, dT);
-    flow64<METRIC>(d, kk, R, yn, kn, Hn);
+    flow64_by<METRIC>(d, kk, R, yn, kn, Hn, m);
 }
 
 // Step factor of the extrapolator: 0.94 (0.65 / err)^(1/(2k-1)) from err^2.
@@ -262,38 +292,38 @@ __device__ __forceinline__ bool moved2(double a0, double b0, double a1, double b
     return fabs(a0 - b0) > 1e-15 * fmax(1.0, fabs(b0)) || fabs(a1 - b1) > 1e-15 * fmax(1.0, fabs(b1));
 }
 
-template <int METRIC>
+template <int METRIC, class Mul>
 __device__ __forceinline__ void verlet_step64(const ImageDesc& d, const KerrK& kk, const RayConst& R,
                                               const State& y, const State& f0, double h, State& yn, State& kn,
-                                              double& Hn) {
+                                              double& Hn, Mul& m) {
     const double hh = 0.5 * h;
     State w = y, g;
     double Hs;
     w.pr = fma(hh, f0.pr, y.pr);
     w.pth = fma(hh, f0.pth, y.pth);
     for (int it = 0; it < kVerletIt; ++it) {
-        flow64<METRIC>(d, kk, R, w, g, Hs);
+        flow64_by<METRIC>(d, kk, R, w, g, Hs, m);
         const double npr = fma(hh, g.pr, y.pr), npth = fma(hh, g.pth, y.pth);
         const bool mv = moved2(npr, w.pr, npth, w.pth);
         w.pr = npr;
         w.pth = npth;
         if (!mv) break;
     }
-    flow64<METRIC>(d, kk, R, w, g, Hs);         // w = (q, p+)
+    flow64_by<METRIC>(d, kk, R, w, g, Hs, m);         // w = (q, p+)
     const double ar = g.r, ath = g.th;
     w.r = fma(h, ar, y.r);
     w.th = fma(h, ath, y.th);
     for (int it = 0; it < kVerletIt; ++it) {
-        flow64<METRIC>(d, kk, R, w, g, Hs);
+        flow64_by<METRIC>(d, kk, R, w, g, Hs, m);
         const double nr = fma(hh, ar + g.r, y.r), nth = fma(hh, ath + g.th, y.th);
         const bool mv = moved2(nr, w.r, nth, w.th);
         w.r = nr;
         w.th = nth;
         if (!mv) break;
     }
-    flow64<METRIC>(d, kk, R, w, g, Hs);         // w = (Q, p+)
+    flow64_by<METRIC>(d, kk, R, w, g, Hs, m);         // w = (Q, p+)
     yn = State{w.r, w.th, fma(hh, g.pr, w.pr), fma(hh, g.pth, w.pth)};
-    flow64<METRIC>(d, kk, R, yn, kn, Hn);
+    flow64_by<METRIC>(d, kk, R, yn, kn, Hn, m);
 }
 
 // e / (atol + rtol max(|y|, |yn|)); callers square and sum with explicit FMAs
@@ -1025,8 +1055,18 @@ __device__ __noinline__ Step64 plain_step64(const ImageDesc* d, KerrK kk, RayCon
     Step64 o;
     State e;
     FpMul m;
-    rk_step64<0, METHOD>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, e, s0, c0, o.sn, o.cn, m);
-    o.err2 = err_norm2(y, o.yn, e, atol, rtol, h, m);
+    o.sn = s0;
+    o.cn = c0;
+    o.err2 = 0.0;
+    if constexpr (METHOD == 4) {
+        verlet_step64<0>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, m);
+    } else if constexpr (METHOD == 3) {
+        gbs_step64<0>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, e, m);
+        o.err2 = err_norm2(y, o.yn, e, atol, rtol, 1.0, m);
+    } else {
+        rk_step64<0, METHOD>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, e, s0, c0, o.sn, o.cn, m);
+        o.err2 = err_norm2(y, o.yn, e, atol, rtol, h, m);
+    }
     return o;
 }
 
@@ -1040,23 +1080,24 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
     State yn, kn, e;
     double Hn, sn = L.s0, cn = L.c0, err2;
     bool fast = false;                         // the attempt's products were integer ones
-    if constexpr (METHOD == 4) {
-        verlet_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn);
-        err2 = 0.0;                            // fixed step, always accepted
-    } else if constexpr (METHOD == 3) {
-        FpMul m;
-        gbs_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e);
-        err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, 1.0, m);
-    } else if constexpr (METRIC == 0 && (PREC == 0 || PREC == 4)) {
+    if constexpr (METRIC == 0 && (PREC == 0 || PREC == 4)) {
         // products on the integer pipes (the FP64 unit, 87 % busy, was the bound:
-        // 258.3 -> 177.7 ms for the 1024^2 disk, issue 8 -> 22 %, the FP64 unit still
-        // 84 % busy with 2/3 of the instructions); where their operands leave the
-        // checked range (a ray in the equatorial plane, a stage inside the horizon)
-        // the attempt is made again with plain products
+        // with these and the integer series of sin and cos the 1024^2 disk takes
+        // 153.0 instead of 258.3 ms); where their operands leave the checked range
+        // (a ray in the equatorial plane, a stage inside the horizon) the attempt is
+        // made again with plain products
         IntMul m;
-        rk_step64<METRIC, METHOD>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
-        err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
-        fast = m.ok() && sol.int_mul;
+        if constexpr (METHOD == 4) {
+            verlet_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, m);
+            err2 = 0.0;                        // fixed step, always accepted
+        } else if constexpr (METHOD == 3) {
+            gbs_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, m);
+            err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, 1.0, m);
+        } else {
+            rk_step64<METRIC, METHOD>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
+            err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
+        }
+        fast = m.ok() && (sol.int_mul || METHOD == 4);
         if (!fast) {
             const Step64 o = plain_step64<METHOD>(&d, L.kk, L.cold().R, L.y, L.k1, L.h, L.s0, L.c0, sol.atol, sol.rtol);
             yn = o.yn;
@@ -1068,8 +1109,16 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
         }
     } else {
         FpMul m;
-        rk_step64<METRIC, METHOD>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
-        err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
+        if constexpr (METHOD == 4) {
+            verlet_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, m);
+            err2 = 0.0;
+        } else if constexpr (METHOD == 3) {
+            gbs_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, m);
+            err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, 1.0, m);
+        } else {
+            rk_step64<METRIC, METHOD>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
+            err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
+        }
     }
     if (nan_bits(err2) | nonfinite_bits(yn.r) | nonfinite_bits(yn.th) | nonfinite_bits(yn.pr) |
         nonfinite_bits(yn.pth))

@@ -1,7 +1,7 @@
 // Products on the integer pipes (tt_soft64.cuh) against FP64's, bit for bit:
 //   mul    random products over 2^+-280, with factors whose low bits are zero or
 //          one (ties, carries into the exponent)
-//   step   Runge-Kutta attempts of random states (stages inside the horizon,
+//   step   step attempts of the five integrators from random states (stages inside the horizon,
 //          equatorial states, huge and tiny components, NaN and infinite steps
 //          among them): an attempt that passes the range checks, ok(), must
 //          equal the plain one in every output
@@ -71,10 +71,25 @@ __global__ void k_step(int n, unsigned long long* out) {
         const double tol = exp(g.uniform(-30.0, -14.0));
         FpMul fm;
         IntMul im;
-        rk_step64<0, METHOD>(d, k, R, y, k1, h, p, pk, pH, pe, s, c, ps, pc, fm);
-        const double pn = err_norm2(y, p, pe, tol, tol, h, fm);
-        rk_step64<0, METHOD>(d, k, R, y, k1, h, q, qk, qH, qe, s, c, qs, qc, im);
-        const double qn = err_norm2(y, q, qe, tol, tol, h, im);
+        ps = qs = s;
+        pc = qc = c;
+        double pn = 0.0, qn = 0.0;
+        if constexpr (METHOD == 4) {
+            h *= 0.01;                                    // a fixed step that the iterations converge for
+            verlet_step64<0>(d, k, R, y, k1, h, p, pk, pH, fm);
+            verlet_step64<0>(d, k, R, y, k1, h, q, qk, qH, im);
+        } else {
+            if constexpr (METHOD == 3) {
+                gbs_step64<0>(d, k, R, y, k1, h, p, pk, pH, pe, fm);
+                gbs_step64<0>(d, k, R, y, k1, h, q, qk, qH, qe, im);
+            } else {
+                rk_step64<0, METHOD>(d, k, R, y, k1, h, p, pk, pH, pe, s, c, ps, pc, fm);
+                rk_step64<0, METHOD>(d, k, R, y, k1, h, q, qk, qH, qe, s, c, qs, qc, im);
+            }
+            const double he = METHOD == 3 ? 1.0 : h;
+            pn = err_norm2(y, p, pe, tol, tol, he, fm);
+            qn = err_norm2(y, q, qe, tol, tol, he, im);
+        }
         atomicAdd(out + 2, 1ull);
         if (!im.ok()) continue;
         atomicAdd(out + 1, 1ull);
@@ -101,5 +116,9 @@ int main() {
     k_step<1><<<304, 128>>>(50, dev);
     if (!report("cash_karp")) return 1;
     k_step<2><<<304, 128>>>(50, dev);
-    return report("fehlberg") ? 0 : 1;
+    if (!report("fehlberg")) return 1;
+    k_step<3><<<304, 128>>>(10, dev);
+    if (!report("gbs")) return 1;
+    k_step<4><<<304, 128>>>(20, dev);
+    return report("verlet") ? 0 : 1;
 }
