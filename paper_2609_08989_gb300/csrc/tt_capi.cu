@@ -160,6 +160,8 @@ int make_desc(const tt_metric* m, const tt_observer* obs, const tt_camera* cam, 
         d->u0 = std::log(t->r_min);
         d->du = (std::log(t->r_max) - d->u0) / (double)(t->nr - 1);
         d->dth = M_PI / (double)(t->nth - 1);
+        d->idu = 1.0 / d->du;
+        d->idth = 1.0 / d->dth;
         d->u0_df = split_df(d->u0);
         d->idu_df = split_df(1.0 / d->du);
         d->idth_df = split_df(1.0 / d->dth);

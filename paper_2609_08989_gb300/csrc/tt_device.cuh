@@ -349,17 +349,51 @@ __device__ __forceinline__ void horner_d(double c0, double c1, double c2, double
     dp = d;
 }
 
-// All five fields (g_tt, g_tphi, g_thth, g_phiphi, g^rr) with d/dr and d/dth.
-__device__ __forceinline__ void table_fields64(const ImageDesc& d, double r, double th,
-                                               double f[5], double fr[5], double ft[5]) {
-    double tu = (log(r) - d.u0) / d.du;
-    double tw = th / d.dth;
-    int k = (int)floor(tu), j = (int)floor(tw);
-    k = min(max(k, 0), d.nr - 2);
-    j = min(max(j, 0), d.nth - 2);
-    const double t = tu - (double)k, w = tw - (double)j;
+// a / b, rounded as the division rounds it, from y = 1 / b rounded: two
+// corrections of a y by the exact remainder (Markstein, IBM J. Res. Dev. 34,
+// 1990: the first leaves less than an ulp of error, the second the rounded
+// quotient).  5 FP64 slots against ~9 for the division.
+__device__ __forceinline__ double div_by(double a, double b, double y) {
+    double q = a * y;
+    q = fma(fma(-q, b, a), y, q);
+    return fma(fma(-q, b, a), y, q);
+}
+
+// floor(x) clamped to [0, n_max] (0 for a NaN), and the same as a double: from
+// the bits of x below 2^21 (a conversion takes as long as a multiply-add, and
+// floor, to int and back were three).
+__device__ __forceinline__ int table_cell(double x, int n_max, double& f) {
+    const int hi = __double2hiint(x), e = (hi >> 20) - 1023;
+    if (hi < 0x3ff00000) {                       // below 1
+        f = 0.0;
+        return 0;
+    }
+    if (e <= 20) {
+        const int k = ((hi & 0xfffff) | 0x100000) >> (20 - e);
+        if (k <= n_max) {
+            f = __hiloint2double(hi & (int)(0xffffffffu << (20 - e)), 0);
+            return k;
+        }
+    }
+    const int k = min(max((int)floor(x), 0), n_max);
+    f = (double)k;
+    return k;
+}
+
+// All five fields (g_tt, g_tphi, g_thth, g_phiphi, g^rr) with d/dr and d/dth;
+// idu, idth: 1 / du and 1 / dth, rounded.  Products by m (tt_soft64.cuh): a
+// derivative may be exactly zero (g_tphi without spin).
+template <class Mul>
+__device__ __forceinline__ void table_fields64(const ImageDesc& d, double idu, double idth, double r, double th,
+                                               double f[5], double fr[5], double ft[5], Mul& m) {
+    m.see(r);
+    const double tu = div_by(log(r) - d.u0, d.du, idu);
+    const double tw = div_by(th, d.dth, idth);
+    double kf, jf;
+    const int k = table_cell(tu, d.nr - 2, kf), j = table_cell(tw, d.nth - 2, jf);
+    const double t = tu - kf, w = tw - jf;
     const double* cell = d.table + ((size_t)j * (d.nr - 1) + k) * kTableCoef;
-    const double inv_dur = 1.0 / (d.du * r), inv_dth = 1.0 / d.dth;
+    const double inv_dur = 1.0 / (d.du * r);
 #pragma unroll
     for (int fi = 0; fi < 5; ++fi) {
         const double2* c = reinterpret_cast<const double2*>(cell + 16 * fi);
@@ -373,37 +407,52 @@ __device__ __forceinline__ void table_fields64(const ImageDesc& d, double r, dou
         horner_d(P[0], P[1], P[2], P[3], t, v, vt);
         const double vw = fma(fma(fma(Q[3], t, Q[2]), t, Q[1]), t, Q[0]);
         f[fi] = v;
-        fr[fi] = vt * inv_dur;
-        ft[fi] = vw * inv_dth;
+        fr[fi] = m.mulz(vt, inv_dur);
+        ft[fi] = m.mulz(vw, idth);
     }
+}
+
+__device__ __forceinline__ void table_fields64(const ImageDesc& d, double r, double th,
+                                               double f[5], double fr[5], double ft[5]) {
+    FpMul m;
+    table_fields64(d, 1.0 / d.du, 1.0 / d.dth, r, th, f, fr, ft, m);
 }
 
 // Flow of H = 1/2 [W/D + g^rr p_r^2 + p_th^2 / g_thth], with the inverse of the
 // (t, phi) block, D = g_tt g_phiphi - g_tphi^2,
-// W = g_phiphi p_t^2 - 2 g_tphi p_t p_phi + g_tt p_phi^2.
+// W = g_phiphi p_t^2 - 2 g_tphi p_t p_phi + g_tt p_phi^2.  (For IntMul the fields
+// and p_r are checked; g_tphi, p_phi, p_th and derivatives may be zero.)
+template <class Mul>
 __device__ __forceinline__ void table_flow64(const ImageDesc& d, const RayConst& R, const State& y,
-                                             State& f, double& H) {
+                                             State& f, double& H, Mul& m) {
     double F[5], Fr[5], Ft[5];
-    table_fields64(d, y.r, y.th, F, Fr, Ft);
-    const double pt2 = R.pt * R.pt, ptp = 2.0 * R.pt * R.pph;
-    double D = fma(F[0], F[3], -F[1] * F[1]);
+    table_fields64(d, d.idu, d.idth, y.r, y.th, F, Fr, Ft, m);
+    m.see(F[0]);
+    m.see(F[2]);
+    m.see(F[3]);
+    m.see(F[4]);
+    m.see(y.pr);
+    m.see(R.pt);
+    const double pt2 = m.mul(R.pt, R.pt), ptp = m.mulz(R.pph, R.pt2);
+    double D = fma(F[0], F[3], m.neg(m.mulz(F[1], F[1])));
     double iD = rcp64(D);
-    double W = fma(F[3], pt2, fma(-F[1], ptp, F[0] * R.pph2));
-    double WiD = W * iD;
+    double W = fma(F[3], pt2, fma(-F[1], ptp, m.mulz(R.pph2, F[0])));
+    double WiD = m.mulz(W, iD);
     double ith = rcp64(F[2]);
-    double pr2 = y.pr * y.pr, pth2 = y.pth * y.pth;
-    H = 0.5 * (WiD + fma(F[4], pr2, pth2 * ith));
-    double dW_r = fma(Fr[3], pt2, fma(-Fr[1], ptp, Fr[0] * R.pph2));
-    double dD_r = fma(Fr[0], F[3], fma(F[0], Fr[3], -2.0 * F[1] * Fr[1]));
-    double dW_t = fma(Ft[3], pt2, fma(-Ft[1], ptp, Ft[0] * R.pph2));
-    double dD_t = fma(Ft[0], F[3], fma(F[0], Ft[3], -2.0 * F[1] * Ft[1]));
-    double ith2 = ith * ith;
-    double d2H_r = fma(fma(-WiD, dD_r, dW_r), iD, fma(Fr[4], pr2, -Fr[2] * ith2 * pth2));
-    double d2H_t = fma(fma(-WiD, dD_t, dW_t), iD, fma(Ft[4], pr2, -Ft[2] * ith2 * pth2));
-    f.r = F[4] * y.pr;
-    f.th = y.pth * ith;
-    f.pr = -0.5 * d2H_r;
-    f.pth = -0.5 * d2H_t;
+    double pr2 = m.mul(y.pr, y.pr), pth2 = m.chkw(y.pth, y.pth);
+    H = 0.5 * (WiD + fma(F[4], pr2, m.chkw(pth2, ith)));
+    double dW_r = fma(Fr[3], pt2, fma(-Fr[1], ptp, m.mulz(R.pph2, Fr[0])));
+    const double m2F1 = m.mulz(F[1], -2.0);
+    double dD_r = fma(Fr[0], F[3], fma(F[0], Fr[3], m.mulz(m2F1, Fr[1])));
+    double dW_t = fma(Ft[3], pt2, fma(-Ft[1], ptp, m.mulz(R.pph2, Ft[0])));
+    double dD_t = fma(Ft[0], F[3], fma(F[0], Ft[3], m.mulz(m2F1, Ft[1])));
+    double ith2 = m.mul(ith, ith);
+    double d2H_r = fma(fma(-WiD, dD_r, dW_r), iD, fma(Fr[4], pr2, m.chkw(m.mulz(m.neg(Fr[2]), ith2), pth2)));
+    double d2H_t = fma(fma(-WiD, dD_t, dW_t), iD, fma(Ft[4], pr2, m.chkw(m.mulz(m.neg(Ft[2]), ith2), pth2)));
+    f.r = m.mul(F[4], y.pr);
+    f.th = m.mulz(y.pth, ith);
+    f.pr = m.mulz(d2H_r, -0.5);
+    f.pth = m.mulz(d2H_t, -0.5);
 }
 
 __device__ __forceinline__ void table_lower64(const ImageDesc& d, double r, double th, double g[5]) {
@@ -426,7 +475,24 @@ struct FlowT64 {
 
 static __device__ __noinline__ FlowT64 table_flow64_call(const ImageDesc* d, RayConst R, State y) {
     FlowT64 o;
-    table_flow64(*d, R, y, o.f, o.H);
+    FpMul m;
+    table_flow64(*d, R, y, o.f, o.H, m);
+    return o;
+}
+
+// The same with integer products, and its range checks' record.
+struct FlowT64Int {
+    State f;
+    double H;
+    unsigned bad;
+};
+
+static __device__ __noinline__ FlowT64Int table_flow64_int_call(const ImageDesc* d, RayConst R, State y, unsigned bad) {
+    FlowT64Int o;
+    IntMul m;
+    m.bad = bad;
+    table_flow64(*d, R, y, o.f, o.H, m);
+    o.bad = m.bad;
     return o;
 }
 

@@ -43,7 +43,14 @@ struct ImageDesc {
     double r_escape;              // escape_factor * r_obs
     double r_fp64;                // mixed paths: double-float steps below this radius
     double th_pole;               // mixed paths: double-float steps within this angle of the axis
-    double r_plus, r_minus;       // Kerr horizons (mixed path: Delta = (r - r_+)(r - r_-))
+    union {                       // Kerr horizons (mixed path: Delta = (r - r_+)(r - r_-));
+        double r_plus;            // for a table 1 / du and 1 / dth, rounded
+        double idu;
+    };
+    union {
+        double r_minus;
+        double idth;
+    };
     // disk
     double r_in, r_out, mdot;
     double fx0, fa;               // x0 = sqrt(r_isco / M), a / M

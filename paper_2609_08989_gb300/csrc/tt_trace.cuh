@@ -80,6 +80,11 @@ __device__ __forceinline__ void flow64_near(const ImageDesc& d, const KerrK& kk,
     if constexpr (METRIC == 0) {
         sincos_near(y.th, th0, s0, c0, s, c, m);
         kerr_flow64_sc(kk, R, y, s, c, f, H, m);
+    } else if constexpr (METRIC == 1 && Mul::kInt) {
+        const FlowT64Int o = table_flow64_int_call(&d, R, y, m.bad);
+        f = o.f;
+        H = o.H;
+        m.bad = o.bad;
     } else {
         flow64<METRIC>(d, kk, R, y, f, H);
     }
@@ -241,7 +246,7 @@ __device__ __forceinline__ void gbs_core(const State& y, const State& f0, double
     err = sub(T[kGbsK - 1], T[kGbsK - 2]);
 }
 
-// The flow with its products formed by m (closed-form metric; a table's are plain).
+// The flow with its products formed by m.
 template <int METRIC, class Mul>
 __device__ __forceinline__ void flow64_by(const ImageDesc& d, const KerrK& kk, const RayConst& R, const State& y,
                                           State& f, double& H, Mul& m) {
@@ -255,7 +260,8 @@ __device__ __forceinline__ void flow64_by(const ImageDesc& d, const KerrK& kk, c
         sincos(y.th, &s, &c);
         kerr_flow64_sc(kk, R, y, s, c, f, H, m);
     } else {
-        flow64<METRIC>(d, kk, R, y, f, H);
+        double s, c;
+        flow64_near<METRIC>(d, kk, R, y, 0.0, 0.0, 1.0, f, H, s, c, m);
     }
 }
 
@@ -1042,14 +1048,14 @@ __device__ __forceinline__ void note_crossing(Lane& L, const State& y, const Sol
     L.pend = true;
 }
 
-// A closed-form Kerr step attempt with plain FP64 products, out of line (the few
+// A step attempt with plain FP64 products, out of line (the few
 // attempts whose products the integer pipes do not take).
 struct Step64 {
     State yn, kn;
     double Hn, sn, cn, err2;
 };
 
-template <int METHOD>
+template <int METRIC, int METHOD>
 __device__ __noinline__ Step64 plain_step64(const ImageDesc* d, KerrK kk, RayConst R, State y, State k1, double h,
                                             double s0, double c0, double atol, double rtol) {
     Step64 o;
@@ -1059,12 +1065,12 @@ __device__ __noinline__ Step64 plain_step64(const ImageDesc* d, KerrK kk, RayCon
     o.cn = c0;
     o.err2 = 0.0;
     if constexpr (METHOD == 4) {
-        verlet_step64<0>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, m);
+        verlet_step64<METRIC>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, m);
     } else if constexpr (METHOD == 3) {
-        gbs_step64<0>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, e, m);
+        gbs_step64<METRIC>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, e, m);
         o.err2 = err_norm2(y, o.yn, e, atol, rtol, 1.0, m);
     } else {
-        rk_step64<0, METHOD>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, e, s0, c0, o.sn, o.cn, m);
+        rk_step64<METRIC, METHOD>(*d, kk, R, y, k1, h, o.yn, o.kn, o.Hn, e, s0, c0, o.sn, o.cn, m);
         o.err2 = err_norm2(y, o.yn, e, atol, rtol, h, m);
     }
     return o;
@@ -1080,7 +1086,7 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
     State yn, kn, e;
     double Hn, sn = L.s0, cn = L.c0, err2;
     bool fast = false;                         // the attempt's products were integer ones
-    if constexpr (METRIC == 0 && (PREC == 0 || PREC == 4)) {
+    if constexpr (METRIC != 2 && (PREC == 0 || PREC == 4)) {
         // products on the integer pipes (the FP64 unit, 87 % busy, was the bound:
         // with these and the integer series of sin and cos the 1024^2 disk takes
         // 153.0 instead of 258.3 ms); where their operands leave the checked range
@@ -1099,7 +1105,7 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
         }
         fast = m.ok() && (sol.int_mul || METHOD == 4);
         if (!fast) {
-            const Step64 o = plain_step64<METHOD>(&d, L.kk, L.cold().R, L.y, L.k1, L.h, L.s0, L.c0, sol.atol, sol.rtol);
+            const Step64 o = plain_step64<METRIC, METHOD>(&d, L.kk, L.cold().R, L.y, L.k1, L.h, L.s0, L.c0, sol.atol, sol.rtol);
             yn = o.yn;
             kn = o.kn;
             Hn = o.Hn;
