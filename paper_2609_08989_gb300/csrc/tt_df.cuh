@@ -194,6 +194,168 @@ __device__ __forceinline__ DF df_rcp(DF x) {
 }
 
 // ---------------------------------------------------------------------------
+// Two double-floats at a time: the same operations on packed FP32 pairs
+// (add/mul/fma.f32x2, sm_100 and later), each half rounded exactly as the scalar
+// instruction rounds it.  A packed instruction does the work of two in one issue
+// slot and half the code: per step attempt of the closed-form kernel 4104
+// instructions instead of 5131 (4700 of them were FP32 additions and
+// multiplications), of the table kernel 13.7 k instead of 17.3 k.  The FP32 pipe
+// itself is no faster (a packed instruction holds it for two cycles), so the
+// gain is in what instruction fetch and issue held up: 512^2 table image 337 ->
+// 296 ms, a 97 x 61 mixed preview (one warp per scheduler) 4.4 -> 4.0 ms, 1024^2
+// closed form 52.7 -> 51.5 ms.
+//
+// ptxas (CUDA 13.0) contracts a packed product whose only use is a packed sum
+// into a multiply-add although both are written .rn; such products are formed
+// by two scalar multiplications here (df_sincos_pair).
+// ---------------------------------------------------------------------------
+typedef unsigned long long f32x2;
+
+__device__ __forceinline__ f32x2 f2_pack(float a, float b) {
+    f32x2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+
+__device__ __forceinline__ float f2_x(f32x2 v) {
+    return __uint_as_float((unsigned)v);
+}
+
+__device__ __forceinline__ float f2_y(f32x2 v) {
+    return __uint_as_float((unsigned)(v >> 32));
+}
+
+__device__ __forceinline__ f32x2 f2_neg(f32x2 v) { return f2_pack(-f2_x(v), -f2_y(v)); }
+
+__device__ __forceinline__ f32x2 f2_add(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ f32x2 f2_sub(f32x2 a, f32x2 b) { return f2_add(a, f2_neg(b)); }
+
+__device__ __forceinline__ f32x2 f2_mul(f32x2 a, f32x2 b) {
+    f32x2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+
+__device__ __forceinline__ f32x2 f2_fma(f32x2 a, f32x2 b, f32x2 c) {
+    f32x2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// x and y, each a double-float, side by side
+struct DF2 {
+    f32x2 hi, lo;
+    __device__ __forceinline__ DF x() const { return DF{f2_x(hi), f2_x(lo)}; }
+    __device__ __forceinline__ DF y() const { return DF{f2_y(hi), f2_y(lo)}; }
+};
+
+__device__ __forceinline__ DF2 df2(DF x, DF y) { return DF2{f2_pack(x.hi, y.hi), f2_pack(x.lo, y.lo)}; }
+__device__ __forceinline__ DF2 df2(DF x) { return df2(x, x); }
+
+__device__ __forceinline__ DF2 fast_two_sum(f32x2 a, f32x2 b) {
+    const f32x2 s = f2_add(a, b);
+    return DF2{s, f2_sub(b, f2_sub(s, a))};
+}
+
+__device__ __forceinline__ DF2 two_sum(f32x2 a, f32x2 b) {
+    const f32x2 s = f2_add(a, b);
+    const f32x2 bb = f2_sub(s, a);
+    return DF2{s, f2_add(f2_sub(a, f2_sub(s, bb)), f2_sub(b, bb))};
+}
+
+__device__ __forceinline__ DF2 df_add(DF2 x, DF2 y) {
+    const DF2 s = two_sum(x.hi, y.hi);
+    return fast_two_sum(s.hi, f2_add(s.lo, f2_add(x.lo, y.lo)));
+}
+
+__device__ __forceinline__ DF2 df_neg(DF2 x) { return DF2{f2_neg(x.hi), f2_neg(x.lo)}; }
+
+__device__ __forceinline__ DF2 df_add_f(DF2 x, f32x2 y) {
+    const DF2 s = two_sum(x.hi, y);
+    return fast_two_sum(s.hi, f2_add(s.lo, x.lo));
+}
+
+__device__ __forceinline__ DF2 df_mul_lazy(DF2 x, DF2 y) {
+    const f32x2 p = f2_mul(x.hi, y.hi);
+    f32x2 e = f2_fma(x.hi, y.hi, f2_neg(p));
+    e = f2_fma(x.hi, y.lo, e);
+    return DF2{p, f2_fma(x.lo, y.hi, e)};
+}
+
+__device__ __forceinline__ DF2 df_mul(DF2 x, DF2 y) {
+    const DF2 m = df_mul_lazy(x, y);
+    return fast_two_sum(m.hi, m.lo);
+}
+
+__device__ __forceinline__ DF2 df_mul_f(DF2 x, f32x2 y) {
+    const f32x2 p = f2_mul(x.hi, y);
+    f32x2 e = f2_fma(x.hi, y, f2_neg(p));
+    e = f2_fma(x.lo, y, e);
+    return fast_two_sum(p, e);
+}
+
+__device__ __forceinline__ DF2 df_sqr_lazy(DF2 x) {
+    const f32x2 p = f2_mul(x.hi, x.hi);
+    const f32x2 e = f2_fma(x.hi, x.hi, f2_neg(p));
+    return DF2{p, f2_fma(f2_add(x.hi, x.hi), x.lo, e)};
+}
+
+__device__ __forceinline__ DF2 df_fma_lazy(DF2 x, DF2 y, DF2 z) {
+    const DF2 m = df_mul_lazy(x, y);
+    const DF2 s = two_sum(m.hi, z.hi);
+    return DF2{s.hi, f2_add(s.lo, f2_add(m.lo, z.lo))};
+}
+
+__device__ __forceinline__ DF2 df_fma(DF2 x, DF2 y, DF2 z) {
+    const DF2 s = df_fma_lazy(x, y, z);
+    return fast_two_sum(s.hi, s.lo);
+}
+
+__device__ __forceinline__ DF2 df_norm(DF2 x) { return two_sum(x.hi, x.lo); }
+
+// The dot products above, two at a time.
+struct DotAcc2 {
+    f32x2 s, t;
+};
+
+__device__ __forceinline__ f32x2 dot_err(DF2 c, DF2 k, f32x2 p) {
+    return f2_add(f2_fma(c.hi, k.hi, f2_neg(p)), f2_fma(c.hi, k.lo, f2_mul(c.lo, k.hi)));
+}
+
+__device__ __forceinline__ DotAcc2 dot_first(DF2 c, DF2 k) {
+    const f32x2 p = f2_mul(c.hi, k.hi);
+    return DotAcc2{p, dot_err(c, k, p)};
+}
+
+__device__ __forceinline__ DotAcc2 dot_next(DotAcc2 d, DF2 c, DF2 k) {
+    const f32x2 p = f2_mul(c.hi, k.hi);
+    const DF2 s = two_sum(d.s, p);
+    return DotAcc2{s.hi, f2_add(d.t, f2_add(s.lo, dot_err(c, k, p)))};
+}
+
+// (one coefficient for both halves)
+__device__ __forceinline__ DotAcc2 dot_first(DF c, DF2 k) { return dot_first(df2(c), k); }
+__device__ __forceinline__ DotAcc2 dot_next(DotAcc2 d, DF c, DF2 k) { return dot_next(d, df2(c), k); }
+
+__device__ __forceinline__ DF2 dot_end(DotAcc2 d) {
+    const DF2 s = two_sum(d.s, d.t);
+    return fast_two_sum(s.hi, s.lo);
+}
+
+// A state as two pairs: q = (r, theta), p = (p_r, p_theta).
+struct StateDF2 {
+    DF2 q, p;
+};
+
+__device__ __forceinline__ StateDF2 pairs(const StateDF& y) { return StateDF2{df2(y.r, y.th), df2(y.pr, y.pth)}; }
+__device__ __forceinline__ StateDF halves(const StateDF2& y) { return StateDF{y.q.x(), y.q.y(), y.p.x(), y.p.y()}; }
+
+// ---------------------------------------------------------------------------
 // sin and cos of theta in double-float, for any theta (a ray through the polar
 // axis continues with theta outside (0, pi)).  theta = k pi/64 + d with
 // |d| <= pi/128; sin and cos of k pi/64 come from a 128-entry table over one
@@ -243,6 +405,33 @@ __device__ __forceinline__ void df_sincos(DF th, DF& s, DF& c) {
     const DF sk = DF{t.x, t.y}, ck = DF{t.z, t.w};
     s = df_add(df_mul(sk, cd), df_mul(ck, sd));
     c = df_sub(df_mul(ck, cd), df_mul(sk, sd));
+}
+
+// (sin, cos) of df_sincos as a pair, the same bit for bit
+__device__ __forceinline__ DF2 df_sincos_pair(DF th) {
+    constexpr float kInv = (float)(64.0 / 3.14159265358979323846);
+    constexpr DF P = df_const(kPiOver64);
+    constexpr float P2 = (float)(kPiOver64 - (double)P.hi - (double)P.lo);
+    const int k = __float2int_rn(th.hi * kInv);    // |k| < 2^24 keeps k P_hi exact below
+    const float kf = (float)k;
+    // d = theta - k P: k P_hi exactly as p0 + e0 (FMA), k P_lo as p1 + e1
+    const float p0 = __fmul_rn(kf, P.hi), e0 = fmaf(kf, P.hi, -p0);
+    const float p1 = __fmul_rn(kf, P.lo), e1 = fmaf(kf, P.lo, -p1);
+    const float d0 = __fsub_rn(th.hi, p0);         // exact (Sterbenz) for k != 0; theta_hi for k = 0
+    const float tail = (th.lo - e0) - ((p1 + e1) + kf * P2);
+    const DF d = fast_two_sum(d0, tail);
+    const DF q = df_sqr(d);                         // d^2 <= 6.1e-4
+    // sin d = d + d q (-1/6 + q (1/120 - q/5040)), cos d = 1 + q (-1/2 + q (1/24 - q/720))
+    const f32x2 qf = f2_pack(q.hi, q.hi);
+    const f32x2 w = f2_pack(__fmul_rn(q.hi, fmaf(-q.hi, 1.0f / 5040.0f, 1.0f / 120.0f)), __fmul_rn(q.hi, fmaf(-q.hi, 1.0f / 720.0f, 1.0f / 24.0f)));
+    constexpr DF M6 = df_const(-1.0 / 6.0);
+    const DF2 m = df_mul(df2(q), df_add_f(df2(M6, DF{-0.5f, 0.0f}), w));
+    const DF2 scd = df_add(df2(d, DF{1.0f, 0.0f}), df2(df_mul(d, m.x()), m.y()));   // sin d, cos d
+    const float4 t = s_df_tab[k & (kSinCosN - 1)];  // k mod 128 (two's complement)
+    const DF sk = DF{t.x, t.y}, ck = DF{t.z, t.w};
+    const DF sd = scd.x(), cd = scd.y();
+    const DF2 u = df_mul(df2(sk, ck), df2(cd)), v = df_mul(df2(ck, df_neg(sk)), df2(sd));
+    return df_add(u, v);
 }
 
 // ---------------------------------------------------------------------------
@@ -322,6 +511,52 @@ __device__ __forceinline__ void kerr_flow_df(const KerrDF& k, const RayDF& R, co
     H = o.H;
 }
 
+// The same flow, bit for bit, with independent operations of one kind in pairs.
+__device__ __forceinline__ void kerr_flow_pair_body(const KerrDF& k, const RayDF& R, const StateDF2& y, StateDF2& f,
+                                                  DF& H) {
+    const DF2 sc2 = df_sincos_pair(y.q.y());
+    const DF s = sc2.x(), c = sc2.y(), r = y.q.x(), pr = y.p.x(), pth = y.p.y();
+    const DF2 trig2 = df_sqr_lazy(sc2), rp2 = df_sqr_lazy(df2(r, pr));
+    const DF s2 = trig2.x(), c2 = trig2.y(), r2 = rp2.x(), pr2 = rp2.y();
+    const DF2 rm = df_add(df2(r), df_neg(df2(k.twoM, k.M)));             // r - 2M, r - M
+    const DF2 sd = df_fma(df2(k.a2, r), df2(c2, rm.x()), df2(r2, k.a2));
+    const DF Sig = sd.x(), Del = sd.y();
+    const DF2 ak = df_fma(df2(df_add(r2, k.a2), R.a2pt2), df2(R.pt, s2), df2(R.apph, R.c0));
+    const DF A = ak.x();
+    const DF2 m1 = df_mul_lazy(df2(Sig, s), df2(Del, c));                // Sigma Delta, sin cos
+    const DF SD = m1.x(), sc = m1.y();
+    const DF inv = df_rcp(df_norm(df_mul_lazy(SD, s2)));
+    const DF2 isd = df_mul_lazy(df2(inv), df_mul_lazy(df2(Del, Sig), df2(s2)));     // 1/Sigma, 1/Delta
+    const DF iS = isd.x(), iD = isd.y();
+    const DF u = df_mul_lazy(inv, SD);
+    const DF AiD = df_mul(A, iD);
+    const DF2 pu = df_sqr_lazy(df2(pth, u));
+    const DF2 m2 = df_mul_lazy(df2(A, R.pph2), df2(AiD, pu.y()));        // A^2/Delta, p_phi^2/sin^4
+    DF K = df_fma(R.pph2, u, ak.y());
+    K = df_add(K, pu.x());
+    K = df_fma(Del, pr2, K);
+    K = df_sub(K, m2.x());
+    const DF H2 = df_mul(K, iS);
+    H = DF{0.5f * H2.hi, 0.5f * H2.lo};
+    const DF2 qt = df_add(df2(df_sqr_lazy(AiD), R.a2pt2), df2(pr2, df_neg(m2.y())));     // q2, t1
+    const DF2 q1t2 = df_fma(df2(R.pt2, k.a2), df2(AiD, H2), df2(H2, qt.y()));
+    const DF2 m3 = df_mul_lazy(df2(Del, sc), df2(pr, iS));
+    f.q = df_mul(df2(m3.x(), pth), df2(iS));
+    const DF2 m4 = df_mul_lazy(df2(r, rm.y()), df2(q1t2.x(), qt.x()));
+    f.p = df_mul(df2(df_sub(m4.x(), m4.y()), m3.y()), df2(iS, df_neg(q1t2.y())));
+}
+
+struct FlowDF2 {
+    StateDF2 f;
+    DF H;
+};
+
+static __device__ __noinline__ FlowDF2 kerr_flow_pair_call(KerrDF k, RayDF R, StateDF2 y) {
+    FlowDF2 o;
+    kerr_flow_pair_body(k, R, y, o.f, o.H);
+    return o;
+}
+
 // ---------------------------------------------------------------------------
 // Natural logarithm in double-float, table-driven in the manner of Tang (ACM
 // TOMS 16, 1990): x = 2^e m with m in [1, 2) and c = 1 + k/32 the nearest
@@ -379,10 +614,12 @@ __device__ __forceinline__ DF df_log(DF x) {
 // coefficients per cell and field, Horner's rule for the value and both
 // unit-cell derivatives) with double-float coefficients and arithmetic.
 // ---------------------------------------------------------------------------
-// p = c0 + c1 x + c2 x^2 + c3 x^3 and dp = dp/dx (both left unnormalised)
-__device__ __forceinline__ void horner_d_df(DF c0, DF c1, DF c2, DF c3, DF x, DF& p, DF& dp) {
-    DF q = df_fma_lazy(c3, x, c2);
-    DF d = df_fma_lazy(c3, x, q);
+// p = c0 + c1 x + c2 x^2 + c3 x^3 and dp = dp/dx (both left unnormalised), of
+// double-floats or pairs of them
+template <class D>
+__device__ __forceinline__ void horner_d_df(D c0, D c1, D c2, D c3, D x, D& p, D& dp) {
+    D q = df_fma_lazy(c3, x, c2);
+    D d = df_fma_lazy(c3, x, q);
     q = df_fma_lazy(q, x, c1);
     d = df_fma_lazy(d, x, q);
     p = df_fma_lazy(q, x, c0);
@@ -418,17 +655,24 @@ __device__ __forceinline__ void table_fields_df(const ImageDesc& d, DF r, DF th,
 #pragma unroll 1
     for (int fi = 0; fi < 5; ++fi) {
         const float4* c = reinterpret_cast<const float4*>(cell + 16 * fi);
-        DF P[4], Q[4];        // sum_j c_ij w^j and its w-derivative, per power i of t
+        DF2 P[2], Q[2];       // sum_j c_ij w^j and its w-derivative, for the powers (i, i + 1) of t
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const float4 a = __ldg(c + 2 * i), b = __ldg(c + 2 * i + 1);
-            horner_d_df(DF{a.x, a.y}, DF{a.z, a.w}, DF{b.x, b.y}, DF{b.z, b.w}, w, P[i], Q[i]);
+        for (int i = 0; i < 2; ++i) {
+            const float4 a = __ldg(c + 4 * i), b = __ldg(c + 4 * i + 1);
+            const float4 e = __ldg(c + 4 * i + 2), g = __ldg(c + 4 * i + 3);
+            horner_d_df(df2(DF{a.x, a.y}, DF{e.x, e.y}), df2(DF{a.z, a.w}, DF{e.z, e.w}),
+                        df2(DF{b.x, b.y}, DF{g.x, g.y}), df2(DF{b.z, b.w}, DF{g.z, g.w}), df2(w), P[i], Q[i]);
         }
-        DF v, vt;
-        horner_d_df(P[0], P[1], P[2], P[3], t, v, vt);
-        const DF vw = df_fma_lazy(df_fma_lazy(df_fma_lazy(Q[3], t, Q[2]), t, Q[1]), t, Q[0]);
-        v = df_norm(v);
-        const DF vr = df_mul(df_norm(vt), inv_dur), vth = df_mul(df_norm(vw), idth);
+        // the value's chain in t beside that of the w-derivative
+        const DF2 t2 = df2(t);
+        DF2 vq = df_fma_lazy(df2(P[1].y(), Q[1].y()), t2, df2(P[1].x(), Q[1].x()));
+        DF vt = df_fma_lazy(P[1].y(), t, vq.x());
+        vq = df_fma_lazy(vq, t2, df2(P[0].y(), Q[0].y()));
+        vt = df_fma_lazy(vt, t, vq.x());
+        vq = df_fma_lazy(vq, t2, df2(P[0].x(), Q[0].x()));
+        const DF v = df_norm(vq.x());
+        const DF2 vd = df_mul(df_norm(df2(vt, vq.y())), df2(inv_dur, idth));
+        const DF vr = vd.x(), vth = vd.y();
         out[(3 * fi) * kDfBlock] = make_float2(v.hi, v.lo);
         out[(3 * fi + 1) * kDfBlock] = make_float2(vr.hi, vr.lo);
         out[(3 * fi + 2) * kDfBlock] = make_float2(vth.hi, vth.lo);
@@ -445,56 +689,63 @@ __device__ __forceinline__ void table_fields_df(const ImageDesc& d, DF r, DF th,
 // The flow of table_flow64 in double-float: H = 1/2 [W/D + g^rr p_r^2 +
 // p_th^2 / g_thth] with D = g_tt g_phiphi - g_tphi^2 and
 // W = g_phiphi p_t^2 - 2 g_tphi p_t p_phi + g_tt p_phi^2.
-__device__ __forceinline__ void table_flow_df(const ImageDesc& d, const RayDF& R, const StateDF& y, StateDF& f,
+__device__ __forceinline__ void table_flow_df(const ImageDesc& d, const RayDF& R, const StateDF2& y, StateDF2& f,
                                               DF& H) {
     DF F[5], Fr[5], Ft[5];
-    table_fields_df(d, y.r, y.th, F, Fr, Ft);
+    const DF pr = y.p.x(), pth = y.p.y();
+    table_fields_df(d, y.q.x(), y.q.y(), F, Fr, Ft);
     const DF D = df_sub(df_mul(F[0], F[3]), df_sqr(F[1]));
     const DF iD = df_rcp(D);
     const DF W = dot_end(dot_next(dot_next(dot_first(F[3], R.ptsq), df_neg(F[1]), R.ptp), F[0], R.pph2));
-    const DF WiD = df_mul(W, iD);
     const DF ith = df_rcp(F[2]);
-    const DF pr2 = df_sqr(y.pr);
-    const DF pthi = df_mul(y.pth, ith);                      // p_th / g_thth
-    const DF pth2i = df_mul(y.pth, pthi);
+    const DF2 m1 = df_mul(df2(W, pth), df2(iD, ith));
+    const DF WiD = m1.x(), pthi = m1.y();                    // W / D, p_th / g_thth
+    const DF pr2 = df_sqr(pr);
+    const DF pth2i = df_mul(pth, pthi);
     const DF H2 = df_add(WiD, df_fma(F[4], pr2, pth2i));
     H = DF{0.5f * H2.hi, 0.5f * H2.lo};
     const DF pthi2 = df_sqr(pthi);                           // p_th^2 / g_thth^2
-    // d(2H)/dx = (dW - W/D dD)/D + d(g^rr) p_r^2 - d(g_thth) p_th^2 / g_thth^2
-#define TT_D2H(G)                                                                                            \
-    df_add(df_mul(df_sub(dot_end(dot_next(dot_next(dot_first(G[3], R.ptsq), df_neg(G[1]), R.ptp), G[0], R.pph2)), \
-                         df_mul(WiD, dot_end(dot_next(dot_next(dot_first(G[0], F[3]), F[0], G[3]),                \
-                                                      DF{-2.0f * F[1].hi, -2.0f * F[1].lo}, G[1])))),           \
-                  iD),                                                                                         \
-           df_sub(df_mul(G[4], pr2), df_mul(G[2], pthi2)))
-    const DF d2H_r = TT_D2H(Fr);
-    const DF d2H_t = TT_D2H(Ft);
-#undef TT_D2H
-    f.r = df_mul(F[4], y.pr);
-    f.th = pthi;
-    f.pr = DF{-0.5f * d2H_r.hi, -0.5f * d2H_r.lo};
-    f.pth = DF{-0.5f * d2H_t.hi, -0.5f * d2H_t.lo};
+    // d(2H)/dx = (dW - W/D dD)/D + d(g^rr) p_r^2 - d(g_thth) p_th^2 / g_thth^2, for x = (r, theta)
+    DF2 G[5];
+#pragma unroll
+    for (int i = 0; i < 5; ++i) G[i] = df2(Fr[i], Ft[i]);
+    const DF2 dW = dot_end(
+        dot_next(dot_next(dot_first(G[3], df2(R.ptsq)), df_neg(G[1]), df2(R.ptp)), G[0], df2(R.pph2)));
+    const DF2 dD = dot_end(dot_next(dot_next(dot_first(G[0], df2(F[3])), F[0], G[3]),
+                                    DF{-2.0f * F[1].hi, -2.0f * F[1].lo}, G[1]));
+    const DF2 d2H =
+        df_add(df_mul(df_add(dW, df_neg(df_mul(df2(WiD), dD))), df2(iD)),
+               df_add(df_mul(G[4], df2(pr2)), df_neg(df_mul(G[2], df2(pthi2)))));
+    f.q = df2(df_mul(F[4], pr), pthi);
+    const f32x2 mh = f2_pack(-0.5f, -0.5f);
+    f.p = DF2{f2_mul(mh, d2H.hi), f2_mul(mh, d2H.lo)};
 }
 
 // One out-of-line copy (descriptor by pointer, the rest by value).
-static __device__ __noinline__ FlowDF table_flow_df_call(const ImageDesc* d, RayDF R, StateDF y) {
-    FlowDF o;
+static __device__ __noinline__ FlowDF2 table_flow_df_call(const ImageDesc* d, RayDF R, StateDF2 y) {
+    FlowDF2 o;
     table_flow_df(*d, R, y, o.f, o.H);
     return o;
 }
 
-// METRIC 0: closed-form Kerr, 1: table.
+// The flow in pairs.  METRIC 0: closed-form Kerr, 1: table.
 template <int METRIC>
-__device__ __forceinline__ void flow_df(const ImageDesc& d, const KerrDF& k, const RayDF& R, const StateDF& y,
-                                        StateDF& f, DF& H) {
+__device__ __forceinline__ void flow_df(const ImageDesc& d, const KerrDF& k, const RayDF& R, const StateDF2& y,
+                                        StateDF2& f, DF& H) {
     static_assert(METRIC == 0 || METRIC == 1, "the double-float kernels take one metric kind per launch");
-    if constexpr (METRIC == 0) {
-        kerr_flow_df(k, R, y, f, H);
-    } else {
-        const FlowDF o = table_flow_df_call(&d, R, y);
-        f = o.f;
-        H = o.H;
-    }
+    FlowDF2 o;
+    if constexpr (METRIC == 0) o = kerr_flow_pair_call(k, R, y);
+    else o = table_flow_df_call(&d, R, y);
+    f = o.f;
+    H = o.H;
+}
+
+// The closed-form flow by component (the mixed paths' zone steps).
+template <int METRIC>
+__device__ __forceinline__ void flow_df(const ImageDesc&, const KerrDF& k, const RayDF& R, const StateDF& y,
+                                        StateDF& f, DF& H) {
+    static_assert(METRIC == 0, "closed-form Kerr");
+    kerr_flow_df(k, R, y, f, H);
 }
 
 }  // namespace tt

@@ -1382,6 +1382,29 @@ __device__ __forceinline__ int step_zone64_split(Lane& L, const SolverDesc& sol)
 // step-size control run in FP32.  ACC 0: the state is the FP64 L.y;
 // ACC 1: the FP32 pair (yhi, L.lo).
 // ---------------------------------------------------------------------------
+// Dormand-Prince weights as double-floats, each part twice (for the packed
+// operations), in constant memory: a21, a31, a32, a41 .. a65, b1, b3 .. b6, e1,
+// e3 .. e7.
+struct Weight2 {
+    float hi[2], lo[2];
+};
+
+constexpr Weight2 weight2(double v) {
+    const DF c = df_const(v);
+    return Weight2{{c.hi, c.hi}, {c.lo, c.lo}};
+}
+
+static __constant__ __align__(16) Weight2 kDpWeights[26] = {
+    weight2(dp::a21), weight2(dp::a31), weight2(dp::a32), weight2(dp::a41), weight2(dp::a42), weight2(dp::a43),
+    weight2(dp::a51), weight2(dp::a52), weight2(dp::a53), weight2(dp::a54), weight2(dp::a61), weight2(dp::a62),
+    weight2(dp::a63), weight2(dp::a64), weight2(dp::a65), weight2(dp::b1),  weight2(dp::b3),  weight2(dp::b4),
+    weight2(dp::b5),  weight2(dp::b6),  weight2(dp::e1),  weight2(dp::e3),  weight2(dp::e4),  weight2(dp::e5),
+    weight2(dp::e6),  weight2(dp::e7)};
+
+__device__ __forceinline__ DF2 dp_weight(int i) {
+    return DF2{*reinterpret_cast<const f32x2*>(kDpWeights[i].hi), *reinterpret_cast<const f32x2*>(kDpWeights[i].lo)};
+}
+
 template <int METRIC, int ACC, bool FULL, class Lane>
 __device__ int step_ray_df(Lane& L, StateF& yhi, const SolverDesc& sol) {
     constexpr int PREC = FULL ? 3 : ACC + 1;
@@ -1409,51 +1432,86 @@ __device__ int step_ray_df(Lane& L, StateF& yhi, const SolverDesc& sol) {
     DF Hs;
     StateDF k1;
     if (!L.kdf_ok) {
-        flow_df<METRIC>(d, kd, rd, y, k1, Hs);
+        if constexpr (FULL) {
+            StateDF2 f;
+            flow_df<METRIC>(d, kd, rd, pairs(y), f, Hs);
+            k1 = halves(f);
+        } else {
+            flow_df<METRIC>(d, kd, rd, y, k1, Hs);
+        }
     } else {
         k1 = StateDF{DF{L.k1f.r, L.k1lo.r}, DF{L.k1f.th, L.k1lo.th}, DF{L.k1f.pr, L.k1lo.pr},
                      DF{L.k1f.pth, L.k1lo.pth}};
     }
-    StateDF k2, k3, k4, k5, k6, k7, ys, yn;
+    StateDF k7, yn;
+    DF Hn;
+    float er, eth, epr, epth;
 #define TT_DS(dst, S)                                                                 \
     ys.r = S(r);                                                                      \
     ys.th = S(th);                                                                    \
     ys.pr = S(pr);                                                                    \
     ys.pth = S(pth);                                                                  \
     flow_df<METRIC>(d, kd, rd, ys, dst, Hs);
+#define TT_DS2(dst, S)                                                                \
+    ys.q = S(q);                                                                      \
+    ys.p = S(p);                                                                      \
+    flow_df<METRIC>(d, kd, rd, ys, dst, Hs);
+    // The error estimate h sum_i e_i k_i is a small difference of nearly equal
+    // stage flows (sum_i e_i = 0): at tolerances near 1e-10 it is formed in
+    // double-float with double-float weights (FULL), else FP32 rounding noise in
+    // it, not the truncation error, would set the step size.
     if constexpr (FULL) {
-        constexpr DF A21 = df_const(a21), A31 = df_const(a31), A32 = df_const(a32);
-        constexpr DF A41 = df_const(a41), A42 = df_const(a42), A43 = df_const(a43);
-        constexpr DF A51 = df_const(a51), A52 = df_const(a52), A53 = df_const(a53), A54 = df_const(a54);
-        constexpr DF A61 = df_const(a61), A62 = df_const(a62), A63 = df_const(a63), A64 = df_const(a64),
-                     A65 = df_const(a65);
-        constexpr DF B1 = df_const(b1), B3 = df_const(b3), B4 = df_const(b4), B5 = df_const(b5), B6 = df_const(b6);
-#define TT_F2(f) df_add(y.f, df_mul_f(df_mul(k1.f, A21), h))
-#define TT_F3(f) df_add(y.f, df_mul_f(dot_end(dot_next(dot_first(A31, k1.f), A32, k2.f)), h))
+        // (r, theta) and (p_r, p_theta) side by side: q and p
+        const StateDF2 y2 = pairs(y), f1 = pairs(k1);
+        const f32x2 h2 = f2_pack(h, h);
+        StateDF2 k2, k3, k4, k5, k6, f7, ys, yn2;
+        const DF2 A21 = dp_weight(0), A31 = dp_weight(1), A32 = dp_weight(2);
+        const DF2 A41 = dp_weight(3), A42 = dp_weight(4), A43 = dp_weight(5);
+        const DF2 A51 = dp_weight(6), A52 = dp_weight(7), A53 = dp_weight(8), A54 = dp_weight(9);
+        const DF2 A61 = dp_weight(10), A62 = dp_weight(11), A63 = dp_weight(12), A64 = dp_weight(13),
+                  A65 = dp_weight(14);
+        const DF2 B1 = dp_weight(15), B3 = dp_weight(16), B4 = dp_weight(17), B5 = dp_weight(18), B6 = dp_weight(19);
+#define TT_F2(f) df_add(y2.f, df_mul_f(df_mul(f1.f, A21), h2))
+#define TT_F3(f) df_add(y2.f, df_mul_f(dot_end(dot_next(dot_first(A31, f1.f), A32, k2.f)), h2))
 #define TT_F4(f) \
-    df_add(y.f, df_mul_f(dot_end(dot_next(dot_next(dot_first(A41, k1.f), A42, k2.f), A43, k3.f)), h))
+    df_add(y2.f, df_mul_f(dot_end(dot_next(dot_next(dot_first(A41, f1.f), A42, k2.f), A43, k3.f)), h2))
 #define TT_F5(f)                                                                                         \
-    df_add(y.f, df_mul_f(dot_end(dot_next(dot_next(dot_next(dot_first(A51, k1.f), A52, k2.f), A53, k3.f), \
-                                          A54, k4.f)), h))
+    df_add(y2.f, df_mul_f(dot_end(dot_next(dot_next(dot_next(dot_first(A51, f1.f), A52, k2.f), A53, k3.f), \
+                                          A54, k4.f)), h2))
 #define TT_F6(f)                                                                                         \
-    df_add(y.f, df_mul_f(dot_end(dot_next(dot_next(dot_next(dot_next(dot_first(A61, k1.f), A62, k2.f),   \
-                                                            A63, k3.f), A64, k4.f), A65, k5.f)), h))
+    df_add(y2.f, df_mul_f(dot_end(dot_next(dot_next(dot_next(dot_next(dot_first(A61, f1.f), A62, k2.f),   \
+                                                            A63, k3.f), A64, k4.f), A65, k5.f)), h2))
 #define TT_F7(f)                                                                                         \
-    df_add(y.f, df_mul_f(dot_end(dot_next(dot_next(dot_next(dot_next(dot_first(B1, k1.f), B3, k3.f),     \
-                                                            B4, k4.f), B5, k5.f), B6, k6.f)), h))
-        TT_DS(k2, TT_F2)
-        TT_DS(k3, TT_F3)
-        TT_DS(k4, TT_F4)
-        TT_DS(k5, TT_F5)
-        TT_DS(k6, TT_F6)
-        yn = StateDF{TT_F7(r), TT_F7(th), TT_F7(pr), TT_F7(pth)};
+    df_add(y2.f, df_mul_f(dot_end(dot_next(dot_next(dot_next(dot_next(dot_first(B1, f1.f), B3, k3.f),     \
+                                                            B4, k4.f), B5, k5.f), B6, k6.f)), h2))
+        TT_DS2(k2, TT_F2)
+        TT_DS2(k3, TT_F3)
+        TT_DS2(k4, TT_F4)
+        TT_DS2(k5, TT_F5)
+        TT_DS2(k6, TT_F6)
+        yn2 = StateDF2{TT_F7(q), TT_F7(p)};
 #undef TT_F2
 #undef TT_F3
 #undef TT_F4
 #undef TT_F5
 #undef TT_F6
 #undef TT_F7
+        flow_df<METRIC>(d, kd, rd, yn2, f7, Hn);
+        const DF2 E1 = dp_weight(20), E3 = dp_weight(21), E4 = dp_weight(22), E5 = dp_weight(23), E6 = dp_weight(24),
+                  E7 = dp_weight(25);
+#define TT_EDF(f)                                                                                       \
+    f2_mul(h2, dot_end(dot_next(dot_next(dot_next(dot_next(dot_next(dot_first(E1, f1.f), E3, k3.f), E4, k4.f), \
+                                                  E5, k5.f), E6, k6.f), E7, f7.f)).hi)
+        const f32x2 eq = TT_EDF(q), ep = TT_EDF(p);
+        er = f2_x(eq);
+        eth = f2_y(eq);
+        epr = f2_x(ep);
+        epth = f2_y(ep);
+#undef TT_EDF
+        yn = halves(yn2);
+        k7 = halves(f7);
     } else {
+        StateDF k2, k3, k4, k5, k6, ys;
 #define TT_G2(f) df_add_f(y.f, h * ((float)a21 * k1.f.hi))
 #define TT_G3(f) df_add_f(y.f, h * fmaf((float)a32, k2.f.hi, (float)a31 * k1.f.hi))
 #define TT_G4(f) df_add_f(y.f, h * fmaf((float)a43, k3.f.hi, fmaf((float)a42, k2.f.hi, (float)a41 * k1.f.hi)))
@@ -1478,36 +1536,18 @@ __device__ int step_ray_df(Lane& L, StateF& yhi, const SolverDesc& sol) {
 #undef TT_G5
 #undef TT_G6
 #undef TT_G7
-    }
-#undef TT_DS
-    DF Hn;
-    flow_df<METRIC>(d, kd, rd, yn, k7, Hn);
-    // The error estimate h sum_i e_i k_i is a small difference of nearly equal
-    // stage flows (sum_i e_i = 0): at tolerances near 1e-10 it is formed in
-    // double-float with double-float weights (FULL), else FP32 rounding noise in
-    // it, not the truncation error, would set the step size.
+        flow_df<METRIC>(d, kd, rd, yn, k7, Hn);
 #define TT_E32(f)                                                                                       \
     h * fmaf((float)e7, k7.f.hi, fmaf((float)e6, k6.f.hi, fmaf((float)e5, k5.f.hi, fmaf((float)e4, k4.f.hi, \
              fmaf((float)e3, k3.f.hi, (float)e1 * k1.f.hi)))))
-#define TT_EDF(f)                                                                                       \
-    (h * dot_end(dot_next(dot_next(dot_next(dot_next(dot_next(dot_first(E1, k1.f), E3, k3.f), E4, k4.f),   \
-                                            E5, k5.f), E6, k6.f), E7, k7.f)).hi)
-    float er, eth, epr, epth;
-    if constexpr (FULL) {
-        constexpr DF E1 = df_const(e1), E3 = df_const(e3), E4 = df_const(e4), E5 = df_const(e5),
-                     E6 = df_const(e6), E7 = df_const(e7);
-        er = TT_EDF(r);
-        eth = TT_EDF(th);
-        epr = TT_EDF(pr);
-        epth = TT_EDF(pth);
-    } else {
         er = TT_E32(r);
         eth = TT_E32(th);
         epr = TT_E32(pr);
         epth = TT_E32(pth);
-    }
 #undef TT_E32
-#undef TT_EDF
+    }
+#undef TT_DS
+#undef TT_DS2
     const float atol = (float)sol.atol, rtol = (float)sol.rtol;
     float err2 = sq_ratio32(er, y.r.hi, yn.r.hi, atol, rtol);
     err2 += sq_ratio32(eth, y.th.hi, yn.th.hi, atol, rtol);
