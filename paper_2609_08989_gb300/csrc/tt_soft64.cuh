@@ -107,6 +107,35 @@ __device__ __forceinline__ Sig53 soft_sub_from(unsigned long long c64, Sig53 a, 
     return o;
 }
 
+// (double)x and (float)x on the integer pipes: a conversion takes an FP64 slot
+// like a multiply-add, and the mixed step of an FP64 state made 14 of them.
+// Zeros, subnormals, infinities and NaNs, and values that a float does not hold
+// as normal numbers, take the conversion.
+__device__ __forceinline__ double int_to_double(float x) {
+    const unsigned u = __float_as_uint(x);
+    double v = __hiloint2double((int)((((u >> 3) & 0x0fffffffu) + (896u << 20)) | (u & 0x80000000u)), (int)(u << 29));
+    if ((u & 0x7f800000u) - 0x00800000u >= 0x7f000000u) v = (double)x;
+    return v;
+}
+
+__device__ __forceinline__ float int_to_float(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
+    // 23 bits of the significand below 9 of the exponent, rounded to nearest even
+    const unsigned a = __funnelshift_l(lo, hi, 3) - (384u << 23);
+    const unsigned up = (a & 1u) + 0x7fffffffu;
+    unsigned r;
+    asm("{\n\t"
+        ".reg .u32 d;\n\t"
+        "add.cc.u32 d, %1, %2;\n\t"
+        "addc.u32 %0, %3, 0;\n\t"
+        "}"
+        : "=r"(r)
+        : "r"(lo << 3), "r"(up), "r"(a));
+    float v = __uint_as_float(r | (hi & 0x80000000u));
+    if ((hi & 0x7ff00000u) - (897u << 20) >= (254u << 20)) v = (float)x;
+    return v;
+}
+
 // How a block of FP64 arithmetic forms its products.
 //   mul(a, b)  the product
 //   chk(a, b)  the product, whose magnitude is to lie in 2^-100 .. 2^100

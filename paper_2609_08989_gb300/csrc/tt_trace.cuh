@@ -1213,10 +1213,11 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
     // only to ~2.4e-7 absolute) sin theta keeps FP32's relative precision, as it
     // does near theta = 0.
     if (ACC == 0) {
-        y = StateF{(float)L.y.r, (float)L.y.th, (float)L.y.pr, (float)L.y.pth};
-        dr0 = (float)(L.y.r - d.r_plus);
+        y = StateF{int_to_float(L.y.r), int_to_float(L.y.th), int_to_float(L.y.pr), int_to_float(L.y.pth)};
+        dr0 = int_to_float(L.y.r - d.r_plus);
         const float m = rintf(y.th * 0.318309886f);
-        dth0 = (float)fma(-(double)m, 3.141592653589793, L.y.th);
+        dth0 = y.th;
+        if (m != 0.0f) dth0 = int_to_float(fma(-int_to_double(m), 3.141592653589793, L.y.th));
     } else {
         y = yhi;
         dr0 = (y.r - L.rph) + (L.lo.r - L.rpl);
@@ -1257,26 +1258,32 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
     StateF yn = {y.r + inc.r, y.th + inc.th, y.pr + inc.pr, y.pth + inc.pth};
     float Hn;
     kerr_flow32(L.f32.Mf, L.f32.a2f, L.f32.rpmf, L.f32.Rf, StateF{yn.r, dth0 + inc.th, yn.pr, yn.pth}, dr0 + inc.r, k7, Hn);
-#define TT_E(f) \
-    h * fmaf((float)e7, k7.f, fmaf((float)e6, k6.f, fmaf((float)e5, k5.f, fmaf((float)e4, k4.f, \
-             fmaf((float)e3, k3.f, (float)e1 * k1.f)))))
+#define TT_ES(f) \
+    fmaf((float)e7, k7.f, fmaf((float)e6, k6.f, fmaf((float)e5, k5.f, fmaf((float)e4, k4.f, \
+         fmaf((float)e3, k3.f, (float)e1 * k1.f)))))
+#define TT_E(f) h * TT_ES(f)
     float err2;
     double err64 = 0.0;
     State y64n;
     if constexpr (PREC == 4) {
         // FP64 norm from the FP32 error terms and the FP64 states
-        y64n = State{L.y.r + (double)inc.r, L.y.th + (double)inc.th, L.y.pr + (double)inc.pr,
-                     L.y.pth + (double)inc.pth};
-        const State e64 = State{(double)TT_E(r), (double)TT_E(th), (double)TT_E(pr), (double)TT_E(pth)};
+        y64n = State{L.y.r + int_to_double(inc.r), L.y.th + int_to_double(inc.th), L.y.pr + int_to_double(inc.pr),
+                     L.y.pth + int_to_double(inc.pth)};
+        const double h64 = int_to_double(h);
+        const State es = State{int_to_double(TT_ES(r)), int_to_double(TT_ES(th)), int_to_double(TT_ES(pr)),
+                               int_to_double(TT_ES(pth))};
         IntMul m;
         m.see(y64n.r);
         m.see(y64n.pr);
+        m.see(h64);
+        const State e64 = State{m.chkw(es.r, h64), m.chkw(es.th, h64), m.chkw(es.pr, h64), m.chkw(es.pth, h64)};
         err64 = err_norm2(L.y, y64n, e64, sol.atol, sol.rtol, 1.0, m);
         if (!(m.ok() && sol.int_mul)) {
             FpMul f;
-            err64 = err_norm2(L.y, y64n, e64, sol.atol, sol.rtol, 1.0, f);
+            const State ef = State{es.r * h64, es.th * h64, es.pr * h64, es.pth * h64};
+            err64 = err_norm2(L.y, y64n, ef, sol.atol, sol.rtol, 1.0, f);
         }
-        err2 = nan_bits(err64) ? __int_as_float(0x7fffffff) : (err64 <= 1.0 ? 0.0f : 2.0f);
+        err2 = nan_bits(err64) ? __int_as_float(0x7fffffff) : (le_pos(err64, 1.0) ? 0.0f : 2.0f);
     } else {
         const float atol = (float)sol.atol, rtol = (float)sol.rtol;
         err2 = sq_ratio32(TT_E(r), y.r, yn.r, atol, rtol);
@@ -1286,6 +1293,7 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
         err2 *= 0.25f;
     }
 #undef TT_E
+#undef TT_ES
 #undef TT_FS
 #undef TT_C2
 #undef TT_C3
@@ -1299,15 +1307,15 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
         bool captured, escaped;
         if (ACC == 0) {
             if constexpr (PREC != 4) {
-                y64n.r = L.y.r + (double)inc.r;
-                y64n.th = L.y.th + (double)inc.th;
-                y64n.pr = L.y.pr + (double)inc.pr;
-                y64n.pth = L.y.pth + (double)inc.pth;
+                y64n.r = L.y.r + int_to_double(inc.r);
+                y64n.th = L.y.th + int_to_double(inc.th);
+                y64n.pr = L.y.pr + int_to_double(inc.pr);
+                y64n.pth = L.y.pth + int_to_double(inc.pth);
             }
-            if (d.disk && ((L.y.th <= kHalfPi) != (y64n.th <= kHalfPi))) note_crossing<0, PREC>(L, L.y, sol);
+            if (d.disk && (le_pos(L.y.th, kHalfPi) != le_pos(y64n.th, kHalfPi))) note_crossing<0, PREC>(L, L.y, sol);
             L.y = y64n;
-            captured = y64n.r < d.r_capture;
-            escaped = y64n.r > d.r_escape;
+            captured = lt_pos(y64n.r, d.r_capture);
+            escaped = lt_pos(d.r_escape, y64n.r);
         } else {
             StateF hi = yhi, lo = L.lo;
             pair_add(hi.r, lo.r, inc.r);
@@ -1331,7 +1339,7 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
         if (captured) return 1;
         if (escaped) return 0;
         if constexpr (PREC == 4) {
-            L.hf = (float)((double)h * fmin(L.last_rej ? 1.0 : 10.0, fmax(0.2, step_factor(err64))));
+            L.hf = int_to_float(next_h(int_to_double(h), err64, L.last_rej ? 1.0 : 10.0));
         } else {
             float fac = (err2 < 1e-30f) ? 10.0f : 0.9f * __powf(err2, -0.1f);
             fac = fminf(L.last_rej ? 1.0f : 10.0f, fmaxf(0.2f, fac));
@@ -1340,7 +1348,7 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
         L.last_rej = false;
     } else {
         L.rejects++;
-        if constexpr (PREC == 4) L.hf = (float)((double)h * fmax(0.2, step_factor(err64)));
+        if constexpr (PREC == 4) L.hf = int_to_float(next_h(int_to_double(h), err64, 1.0));
         else L.hf = h * fmaxf(0.2f, 0.9f * __powf(err2, -0.1f));
         L.last_rej = true;
     }
@@ -1774,8 +1782,8 @@ __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, l
                 // coordinate singularities); the distance to the axis is
                 // |theta - m pi| for the nearest integer m, since a ray through the
                 // axis continues with theta outside (0, pi)
-                const float thf = (ACC == 0) ? (float)L.y.th : yhi.th;
-                const float rf = (ACC == 0) ? (float)L.y.r : yhi.r;
+                const float thf = (ACC == 0) ? int_to_float(L.y.th) : yhi.th;
+                const float rf = (ACC == 0) ? int_to_float(L.y.r) : yhi.r;
                 const float axis = fabsf(fmaf(-rintf(thf * 0.318309886f), 3.14159274f, thf));
                 want64 = (rf < L.fp64f) || (axis < L.thpf);
             }
