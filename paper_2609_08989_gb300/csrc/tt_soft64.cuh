@@ -107,17 +107,25 @@ __device__ __forceinline__ Sig53 soft_sub_from(unsigned long long c64, Sig53 a, 
     return o;
 }
 
-// (double)x and (float)x on the integer pipes: a conversion takes an FP64 slot
-// like a multiply-add, and the mixed step of an FP64 state made 14 of them.
-// Zeros, subnormals, infinities and NaNs, and values that a float does not hold
-// as normal numbers, take the conversion.
+// (double)x for a finite x, on the integer pipes: a conversion takes an FP64 slot
+// like a multiply-add (predicated off too, so no branch around one may be short
+// enough to be predicated).  x below 2^-60 goes through x 2^64, so that subnormals
+// are normal on the way.
 __device__ __forceinline__ double int_to_double(float x) {
-    const unsigned u = __float_as_uint(x);
-    double v = __hiloint2double((int)((((u >> 3) & 0x0fffffffu) + (896u << 20)) | (u & 0x80000000u)), (int)(u << 29));
-    if ((u & 0x7f800000u) - 0x00800000u >= 0x7f000000u) v = (double)x;
-    return v;
+    const bool small = fabsf(x) < 0x1p-60f;
+    const unsigned u = __float_as_uint(small ? x * 0x1p64f : x);
+    const unsigned bias = small ? (896u - 64u) << 20 : 896u << 20;
+    const unsigned hi = (((u >> 3) & 0x0fffffffu) + bias) | (u & 0x80000000u);
+    return __hiloint2double((int)(x == 0.0f ? u : hi), (int)(u << 29));
 }
 
+// Whether int_to_float does not take x: not zero, and outside the normal floats.
+__device__ __forceinline__ bool float_odd(double x) {
+    const unsigned hi = (unsigned)__double2hiint(x);
+    return (hi & 0x7ff00000u) - (897u << 20) >= (254u << 20) && ((hi << 1) | (unsigned)__double2loint(x)) != 0u;
+}
+
+// (float)x for an x that is not odd, on the integer pipes.
 __device__ __forceinline__ float int_to_float(double x) {
     const unsigned hi = (unsigned)__double2hiint(x), lo = (unsigned)__double2loint(x);
     // 23 bits of the significand below 9 of the exponent, rounded to nearest even
@@ -131,9 +139,7 @@ __device__ __forceinline__ float int_to_float(double x) {
         "}"
         : "=r"(r)
         : "r"(lo << 3), "r"(up), "r"(a));
-    float v = __uint_as_float(r | (hi & 0x80000000u));
-    if ((hi & 0x7ff00000u) - (897u << 20) >= (254u << 20)) v = (float)x;
-    return v;
+    return __uint_as_float(((hi << 1) == 0u ? 0u : r) | (hi & 0x80000000u));
 }
 
 // How a block of FP64 arithmetic forms its products.

@@ -1195,6 +1195,20 @@ __device__ __forceinline__ bool pair_below(float hi, float lo, float ch, float c
     return ((hi - ch) + (lo - cl)) < 0.0f;
 }
 
+// (float)x by conversion, out of line (a conversion in line would be predicated).
+static __device__ __noinline__ float float_call(double x) { return (float)x; }
+
+__device__ __forceinline__ float state_float(double x) { return float_odd(x) ? float_call(x) : int_to_float(x); }
+
+struct Floats6 {
+    StateF y;
+    float dr, dth;
+};
+
+static __device__ __noinline__ Floats6 floats6(State y, double dr, double dth) {
+    return Floats6{StateF{(float)y.r, (float)y.th, (float)y.pr, (float)y.pth}, (float)dr, (float)dth};
+}
+
 template <int PREC, class Lane>
 __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
     constexpr int ACC = (PREC == 2) ? 1 : 0;
@@ -1213,11 +1227,20 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
     // only to ~2.4e-7 absolute) sin theta keeps FP32's relative precision, as it
     // does near theta = 0.
     if (ACC == 0) {
-        y = StateF{int_to_float(L.y.r), int_to_float(L.y.th), int_to_float(L.y.pr), int_to_float(L.y.pth)};
-        dr0 = int_to_float(L.y.r - d.r_plus);
-        const float m = rintf(y.th * 0.318309886f);
-        dth0 = y.th;
-        if (m != 0.0f) dth0 = int_to_float(fma(-int_to_double(m), 3.141592653589793, L.y.th));
+        const double dr64 = L.y.r - d.r_plus;
+        const float m = rintf(state_float(L.y.th) * 0.318309886f);
+        const double dth64 = fma(-int_to_double(m), 3.141592653589793, L.y.th);
+        if (float_odd(L.y.r) || float_odd(L.y.th) || float_odd(L.y.pr) || float_odd(L.y.pth) || float_odd(dr64) ||
+            float_odd(dth64)) {
+            const Floats6 o = floats6(L.y, dr64, dth64);
+            y = o.y;
+            dr0 = o.dr;
+            dth0 = o.dth;
+        } else {
+            y = StateF{int_to_float(L.y.r), int_to_float(L.y.th), int_to_float(L.y.pr), int_to_float(L.y.pth)};
+            dr0 = int_to_float(dr64);
+            dth0 = int_to_float(dth64);
+        }
     } else {
         y = yhi;
         dr0 = (y.r - L.rph) + (L.lo.r - L.rpl);
@@ -1339,7 +1362,7 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
         if (captured) return 1;
         if (escaped) return 0;
         if constexpr (PREC == 4) {
-            L.hf = int_to_float(next_h(int_to_double(h), err64, L.last_rej ? 1.0 : 10.0));
+            L.hf = state_float(next_h(int_to_double(h), err64, L.last_rej ? 1.0 : 10.0));
         } else {
             float fac = (err2 < 1e-30f) ? 10.0f : 0.9f * __powf(err2, -0.1f);
             fac = fminf(L.last_rej ? 1.0f : 10.0f, fmaxf(0.2f, fac));
@@ -1348,7 +1371,7 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
         L.last_rej = false;
     } else {
         L.rejects++;
-        if constexpr (PREC == 4) L.hf = int_to_float(next_h(int_to_double(h), err64, 1.0));
+        if constexpr (PREC == 4) L.hf = state_float(next_h(int_to_double(h), err64, 1.0));
         else L.hf = h * fmaxf(0.2f, 0.9f * __powf(err2, -0.1f));
         L.last_rej = true;
     }
@@ -1782,8 +1805,8 @@ __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, l
                 // coordinate singularities); the distance to the axis is
                 // |theta - m pi| for the nearest integer m, since a ray through the
                 // axis continues with theta outside (0, pi)
-                const float thf = (ACC == 0) ? int_to_float(L.y.th) : yhi.th;
-                const float rf = (ACC == 0) ? int_to_float(L.y.r) : yhi.r;
+                const float thf = (ACC == 0) ? state_float(L.y.th) : yhi.th;
+                const float rf = (ACC == 0) ? state_float(L.y.r) : yhi.r;
                 const float axis = fabsf(fmaf(-rintf(thf * 0.318309886f), 3.14159274f, thf));
                 want64 = (rf < L.fp64f) || (axis < L.thpf);
             }
