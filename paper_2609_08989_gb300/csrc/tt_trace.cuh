@@ -571,7 +571,12 @@ struct RayCold {
     RayConst R;
     State yc;               // a disk crossing waiting for its (batched) refinement: the start of its step
     double hmax, inten;
-    double pad;             // 15 doubles: a warp's 64-bit accesses to one field fall in distinct banks
+};
+
+// The double-float constants of a ray in closed-form Kerr.
+struct ZoneDF {
+    KerrDF k;
+    DF pt, apph, pph2, a2pt2, c0, pt2;
 };
 
 // What the FP32 flow needs of a ray: its constants, M, a^2 and r_+ - r_-.
@@ -605,24 +610,47 @@ struct LaneBase {
     StateF k1lo;
     bool kdf_ok;
     float hmaxf;
-    KerrDF kdf;
-    RayDF rdf;
 };
 
 // In registers, or with the cold part in the thread's slot of shared memory (the
 // mixed paths with FP32 control: at 128 registers it would be spilled; 38.7 ->
 // 37.7 ms per 2048^2 image; the prescribed split, whose FP64 zone steps read the
 // constants at every stage, 36.5 -> 37.3 ms per 1024^2 image, keeps registers).
+// The slot also holds the zone steps' double-float constants, which each such
+// step otherwise formed anew by 44 FP64 slots of conversions.
 struct LaneReg : LaneBase {
     RayCold c;
+    KerrDF kdf;
+    RayDF rdf;
     __device__ __forceinline__ RayCold& cold() { return c; }
+    __device__ __forceinline__ void set_df(const KerrDF& k, const RayDF& r) {
+        kdf = k;
+        rdf = r;
+    }
+    __device__ __forceinline__ KerrDF kerr_df() const { return kdf; }
+    __device__ __forceinline__ RayDF ray_df() const { return rdf; }
 };
 
+// 23 doubles: a warp's 64-bit accesses to one field fall in distinct banks.
+struct MixSlot {
+    RayCold c;
+    ZoneDF z;
+};
+static_assert(sizeof(MixSlot) % 16 == 8, "an odd number of doubles");
+
 constexpr int kMixBlock = 256;
-static __shared__ RayCold s_cold[kMixBlock];
+static __shared__ MixSlot s_mix[kMixBlock];
 
 struct LaneShared : LaneBase {
-    __device__ __forceinline__ RayCold& cold() { return s_cold[threadIdx.x]; }
+    __device__ __forceinline__ RayCold& cold() { return s_mix[threadIdx.x].c; }
+    __device__ __forceinline__ void set_df(const KerrDF& k, const RayDF& r) {
+        s_mix[threadIdx.x].z = ZoneDF{k, r.pt, r.apph, r.pph2, r.a2pt2, r.c0, r.pt2};
+    }
+    __device__ __forceinline__ KerrDF kerr_df() const { return s_mix[threadIdx.x].z.k; }
+    __device__ __forceinline__ RayDF ray_df() const {
+        const ZoneDF& z = s_mix[threadIdx.x].z;
+        return RayDF{z.pt, z.apph, z.pph2, z.a2pt2, z.c0, z.pt2, DF{0.0f, 0.0f}, DF{0.0f, 0.0f}};
+    }
 };
 
 // Output stores.  The bounds-checking build (TT_BOUNDS_CHECK) tests every index
@@ -881,11 +909,10 @@ __device__ bool init_ray(Lane& L, const ImageDesc* d_ptr, long long q, const Sol
         L.fp64f = (float)d.r_fp64;
         L.thpf = (float)d.th_pole;
         L.lamf = 0.0f;
+        if (sol.precision != 4 || df_init) L.set_df(make_kerr_df(L.kk), make_ray_df(L.cold().R));
         if (sol.precision == 3 || df_init) {
             // double-float steps: the FP64 path's starting step (once per ray), so
             // that both begin the same step sequence
-            L.kdf = make_kerr_df(L.kk);
-            L.rdf = make_ray_df(L.cold().R);
             double H64;
             flow64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, H64);
             L.cold().hmax = fabs(H64);
@@ -1445,15 +1472,8 @@ __device__ int step_ray_df(Lane& L, StateF& yhi, const SolverDesc& sol) {
     const float hmin = (sol.h_min > 0.0) ? (float)sol.h_min : 1e-14f * fmaxf(1.0f, L.lamf);
     if (h < hmin) return 3;
     using namespace dp;
-    KerrDF kd;
-    RayDF rd;
-    if constexpr (FULL) {
-        kd = L.kdf;
-        rd = L.rdf;
-    } else {
-        kd = make_kerr_df(L.kk);
-        rd = make_ray_df(L.cold().R);
-    }
+    const KerrDF kd = L.kerr_df();
+    const RayDF rd = L.ray_df();
     StateDF y;
     if constexpr (ACC == 0) {
         y = StateDF{df_of(L.y.r), df_of(L.y.th), df_of(L.y.pr), df_of(L.y.pth)};
