@@ -251,13 +251,15 @@ template <int METRIC, class Mul>
 __device__ __forceinline__ void flow64_by(const ImageDesc& d, const KerrK& kk, const RayConst& R, const State& y,
                                           State& f, double& H, Mul& m) {
     if constexpr (METRIC == 0) {
-        double s, c;
+        double s, c, th = y.th;
         if (Mul::kInt) {
             // without sincos's branch for huge angles (they fail the check)
-            m.must(abs_below_hi(y.th, kHi1e5));
-            __builtin_assume(fabs(y.th) < 1e5);
+            const bool near = abs_below_hi(th, kHi1e5);
+            m.must(near);
+            th = near ? th : 0.0;
+            __builtin_assume(fabs(th) < 1e5);
         }
-        sincos(y.th, &s, &c);
+        sincos(th, &s, &c);
         kerr_flow64_sc(kk, R, y, s, c, f, H, m);
     } else {
         double s, c;
@@ -593,6 +595,7 @@ struct LaneBase {
     KerrK kk;
     double h, lam;
     int steps, rejects, ncross, nrec, code;
+    int plain_run;          // FP64 steps: attempts in a row that integer products did not take
     bool last_rej;
     bool pend;              // a crossing is waiting in cold().yc
     // mixed precision
@@ -840,6 +843,7 @@ __device__ bool init_ray(Lane& L, const ImageDesc* d_ptr, long long q, const Sol
     L.cold().hmax = 0.0;
     L.lam = 0.0;
     L.last_rej = false;
+    L.plain_run = 0;
     L.pend = false;
     const long long p = d.pix_begin + q;
     const long long i = p % d.nx, j = p / d.nx;
@@ -1075,6 +1079,8 @@ __device__ __forceinline__ void note_crossing(Lane& L, const State& y, const Sol
     L.pend = true;
 }
 
+constexpr int kPlainRun = 4;
+
 // A step attempt with plain FP64 products, out of line (the few
 // attempts whose products the integer pipes do not take).
 struct Step64 {
@@ -1111,28 +1117,33 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
     const double hmin = (sol.h_min > 0.0) ? sol.h_min : 1e-14 * fmax(1.0, fabs(L.lam));
     if (lt_pos(L.h, hmin)) return 3;
     State yn, kn, e;
-    double Hn, sn = L.s0, cn = L.c0, err2;
+    double Hn, sn = L.s0, cn = L.c0, err2 = 0.0;
     bool fast = false;                         // the attempt's products were integer ones
     if constexpr (METRIC != 2 && (PREC == 0 || PREC == 4)) {
         // products on the integer pipes (the FP64 unit, 87 % busy, was the bound:
         // with these and the integer series of sin and cos the 1024^2 disk takes
-        // 153.0 instead of 258.3 ms); where their operands leave the checked range
-        // (a ray in the equatorial plane, a stage inside the horizon) the attempt is
-        // made again with plain products
-        IntMul m;
-        if constexpr (METHOD == 4) {
-            verlet_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, m);
-            err2 = 0.0;                        // fixed step, always accepted
-        } else if constexpr (METHOD == 3) {
-            gbs_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, m);
-            err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, 1.0, m);
-        } else {
-            rk_step64<METRIC, METHOD>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
-            err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
+        // 152.9 instead of 258.8 ms); where their operands leave the checked range (a
+        // stage inside the horizon) the attempt is made again with plain products,
+        // and a ray whose operands leave it at every attempt (one that stays in the
+        // equatorial plane, p_theta = 0) goes on with plain products alone
+        if ((sol.int_mul || METHOD == 4) && L.plain_run < kPlainRun) {
+            IntMul m;
+            if constexpr (METHOD == 4) {
+                verlet_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, m);
+                err2 = 0.0;                    // fixed step, always accepted
+            } else if constexpr (METHOD == 3) {
+                gbs_step64<METRIC>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, m);
+                err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, 1.0, m);
+            } else {
+                rk_step64<METRIC, METHOD>(d, L.kk, L.cold().R, L.y, L.k1, L.h, yn, kn, Hn, e, L.s0, L.c0, sn, cn, m);
+                err2 = err_norm2(L.y, yn, e, sol.atol, sol.rtol, L.h, m);
+            }
+            fast = m.ok();
+            L.plain_run = fast ? 0 : L.plain_run + 1;
         }
-        fast = m.ok() && (sol.int_mul || METHOD == 4);
         if (!fast) {
-            const Step64 o = plain_step64<METRIC, METHOD>(&d, L.kk, L.cold().R, L.y, L.k1, L.h, L.s0, L.c0, sol.atol, sol.rtol);
+            const Step64 o =
+                plain_step64<METRIC, METHOD>(&d, L.kk, L.cold().R, L.y, L.k1, L.h, L.s0, L.c0, sol.atol, sol.rtol);
             yn = o.yn;
             kn = o.kn;
             Hn = o.Hn;
