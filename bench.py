@@ -73,10 +73,11 @@ METHOD_NAMES = {v: k for k, v in METHODS.items()}
 # its stages, norm and control as in the FP64 step before the h-scaling above).
 FLOPS_PER_STEP_F32 = 6 * 72 + 232 + 20 + 5
 # FP64 thread instructions per Dormand-Prince step attempt of the FP64 kernel, from ncu's
-# instruction counts on the 512^2 image (7.02e7 attempts): DFMA, DMUL, DADD
-FP64_ISSUED_PER_STEP = (260.8, 199.6, 19.5)
-# FP32 thread instructions (FFMA + FMUL + FADD) per double-float step attempt, from ncu's
-# instruction counts on the 512^2 image
+# instruction counts on the 512^2 image (7.02e7 attempts): DFMA, DMUL, DADD (most products
+# and the sine and cosine series of small angle steps run on the integer pipes)
+FP64_ISSUED_PER_STEP = (236.9, 4.7, 29.4)
+# FP32 thread operations (FFMA + FMUL + FADD, a packed instruction as two) per double-float
+# step attempt, from ncu's instruction counts on the 512^2 image
 DF_FP32_INST_PER_STEP = 4693
 # the same for the double-float kernel on the tabulated metric (256^2 image of its scene)
 TABLE_DF_FP32_INST_PER_STEP = 15398
