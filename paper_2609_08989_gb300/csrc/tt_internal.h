@@ -109,6 +109,7 @@ struct TuneParams {
     int fp64_wait;        // mixed: zone steps run after this many iterations of waiting
     int crit_stride;      // mixed: near-critical rays on one SM in crit_stride
     int crit_refill;      // mixed: refill threshold of a warp tracing near-critical rays
+    int outward;          // hand tile rows out from the middle of the image outward
 };
 
 // Images handed to one launch by value (kernel parameters, no host-to-device

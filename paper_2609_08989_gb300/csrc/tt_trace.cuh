@@ -745,18 +745,19 @@ __device__ __forceinline__ long long outward(long long k, long long n, long long
 // per tile), so that the rays a warp takes together start close on the sky and
 // stay in step; others in runs of 32 pixels.
 //
-// OUTWARD: tile rows (or runs) are taken outward from the line beta = 0.  The
+// from_middle: tile rows (or runs) are taken outward from the line beta = 0.  The
 // longest rays, those that circle the hole, pass near it, at most ~7 M away;
 // taken in order of beta they start when half of the image is done, and with few
 // rays per lane the last of them run on a GPU that is otherwise empty: the
 // double-float table image of 512^2 (6.7 rays per lane) 310 -> 268 ms, of 768^2
 // 560 -> 491 ms; FP64 384^2 32.3 -> 29.0 ms, double-float 256^2 6.4 -> 5.3 ms, the
-// prescribed split's 1024^2 35.1 -> 32.2 ms; no change with one ray per lane or
-// with many.  The mixed kernels whose near-critical rays run apart have no such
+// prescribed split's 1024^2 35.1 -> 32.2 ms; no change with many.  Where every ray
+// has a lane from the start there is no order to gain from, and narrow images
+// lost (33 x 299 table 59 -> 63 ms): launches of at most 256 rays per SM keep the
+// order of beta.  The mixed kernels whose near-critical rays run apart have no such
 // tail, and are 2-10 % slower when the rays that need zone steps come all at
 // once (768^2 8.8 -> 9.8 ms, 2048^2 38.1 -> 39.1 ms): they keep the order of beta.
-template <bool OUTWARD>
-__device__ __forceinline__ long long tile_pixel(const ImageDesc& d, long long q) {
+__device__ __forceinline__ long long tile_pixel(const ImageDesc& d, long long q, bool from_middle) {
     const long long band = 4LL * d.nx;
     // the row of beta = 0, within the range (an undefined quotient gives some row)
     const double j0 = fmin(fmax(-d.beta_min / d.dbeta, 0.0), 2147483647.0);
@@ -766,11 +767,11 @@ __device__ __forceinline__ long long tile_pixel(const ImageDesc& d, long long q)
         long long ty = tile / tiles_x;
         const long long tx = tile - ty * tiles_x;
         const int lane = (int)(q & 31);
-        if (OUTWARD) ty = outward(ty, rows, min(max(mid / band, 0LL), rows - 1));
+        if (from_middle) ty = outward(ty, rows, min(max(mid / band, 0LL), rows - 1));
         return (ty * 4 + (lane >> 3)) * d.nx + tx * 8 + (lane & 7);
     }
     const long long runs = d.pix_count >> 5, run = q >> 5;     // (a last part of a run keeps its place)
-    if (!OUTWARD || run >= runs) return q;
+    if (!from_middle || run >= runs) return q;
     return outward(run, runs, min(max(mid >> 5, 0LL), runs - 1)) * 32 + (q & 31);
 }
 
@@ -1772,7 +1773,7 @@ __device__ __forceinline__ void trace_loop(const ImageDesc* descs, int n_desc, l
                     if (rid < total) {
                         const int im = (n_desc == 1) ? 0 : find_image(descs, n_desc, rid);
                         const ImageDesc* dp = descs + im;
-                        const long long q = tile_pixel<OUTWARD>(*dp, rid - dp->ray_begin);
+                        const long long q = tile_pixel(*dp, rid - dp->ray_begin, OUTWARD && tp.outward);
                         const bool skip = MIX && band > 0.0f && near_critical(*dp, q, band);
                         if (!skip && init_ray<METRIC>(L, dp, q, sol)) {
                             st = kRun;
@@ -1920,7 +1921,7 @@ __device__ __forceinline__ void critical_loop(const ImageDesc* descs, int n_desc
                     if (rid < total) {
                         const int im = (n_desc == 1) ? 0 : find_image(descs, n_desc, rid);
                         const ImageDesc* dp = descs + im;
-                        const long long q = tile_pixel<false>(*dp, rid - dp->ray_begin);
+                        const long long q = tile_pixel(*dp, rid - dp->ray_begin, false);
                         if (near_critical(*dp, q, band) && init_ray<0>(L, dp, q, solc, true)) {
                             st = kRun;
                             if (ACC == 1) split_state(L.y, yhi, L.lo);
@@ -2000,6 +2001,7 @@ void fill_params(LaunchParams<N>& p, const ImageDesc* descs, int n, long long to
     p.tune.fp64_wait = shape.fp64_wait > 0 ? shape.fp64_wait : 64;
     p.tune.crit_stride = shape.crit_stride > 0 ? shape.crit_stride : 1;
     p.tune.crit_refill = shape.crit_refill > 0 ? shape.crit_refill : 32;
+    p.tune.outward = total > 256LL * sm_count();      // (see tile_pixel)
     p.total = total;
     p.queue = queue;
     for (int i = 0; i < n; ++i) p.desc[i] = descs[i];

@@ -13,7 +13,8 @@ torch = pytest.importorskip("torch")
 
 # (nx, ny, first pixel, pixels or 0 for the rest): tiles, one tile row, ragged
 # runs, less than one run, a last part of a run; beta = 0 inside, above, below
-RANGES = [(16, 12, 0, 0), (8, 4, 0, 0), (16, 24, 64, 128), (9, 7, 0, 0), (5, 3, 2, 9), (33, 11, 40, 300), (40, 1, 0, 0)]
+RANGES = [(16, 12, 0, 0), (8, 4, 0, 0), (16, 24, 64, 128), (9, 7, 0, 0), (5, 3, 2, 9), (33, 11, 40, 300), (40, 1, 0, 0),
+          (240, 168, 0, 0), (241, 165, 7, 0)]       # more rays than lanes: outward from the middle
 
 
 @pytest.mark.parametrize("precision", [scenes.FP64, scenes.DOUBLE_FLOAT, scenes.MIXED_PAIR])
@@ -25,8 +26,11 @@ def test_every_pixel_once(precision, beta):
     for nx, ny, begin, count in RANGES:
         sc = scenes.kerr_disk(16, precision).replace(nx=nx, ny=ny, beta_min=beta[0], beta_max=beta[1], rtol=1e-8,
                                                      atol=1e-8)
-        # the whole image row by row: each call one range with an order of its own
-        rows = [T.to_numpy(T.trace(sc, pix_begin=j * nx, pix_count=nx)) for j in range(ny)]
+        # the whole image band by band (row by row when small): each call one range
+        # with an order of its own
+        band = nx * max(1, ny // 12)
+        rows = [T.to_numpy(T.trace(sc, pix_begin=p, pix_count=min(band, nx * ny - p)))
+                for p in range(0, nx * ny, band)]
         n = count or nx * ny - begin
         out = T.alloc_outputs(n)
         for v in out.values():
