@@ -91,7 +91,7 @@ BYTES_OUT_PER_PIXEL = 3 * 3 * 8 + 8 + 8 + 4 + 4 + 1 + 1
 TRAFFIC_BYTES_1024 = 2555392 + 51188480
 # host-to-device input of one step: the launch's parameter block (sizeof(tt::LaunchParams<1>):
 # solver settings, launch shape and the image descriptor)
-DESC_BYTES = 728
+DESC_BYTES = 736
 # The tolerance of the equal-accuracy comparison: the mixed paths' own, at which the FP64
 # and double-float paths also keep |H| <= 1e-6 on every escaped ray of the 2048^2 disk
 # image (the next looser ones measured there, 2e-8 and 3e-8, give 1.1e-6 and more) and
