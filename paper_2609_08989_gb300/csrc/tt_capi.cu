@@ -184,6 +184,8 @@ int make_desc(const tt_metric* m, const tt_observer* obs, const tt_camera* cam, 
         d->obs_ir = 1.0 / std::sqrt(g[2]);
         d->obs_ith = 1.0 / std::sqrt(g[3]);
         d->obs_iph = 1.0 / std::sqrt(g[4]);
+        d->cos2_obs = c * c;
+        d->cot2_obs = c * c / s2;
         d->obs_ready = 1;
     }
     d->r_capture = r_h * (1.0 + sol->horizon_eps);

@@ -36,7 +36,15 @@ struct ImageDesc {
     const double* table;          // device patch coefficients, cell-major (see tt_capi.cu)
     const float2* table_df;       // the same as double-float (hi, lo) pairs
     int nr, nth;
-    double u0, du, dth;           // ln r_min, ln-spacing, theta spacing
+    double u0;                    // ln r_min
+    union {                       // a table's ln-spacing and theta spacing; for Kerr cos^2 and
+        double du;                // cos^2 / sin^2 of the observer's theta
+        double cos2_obs;
+    };
+    union {
+        double dth;
+        double cot2_obs;
+    };
     float2 u0_df, idu_df, idth_df;          // u0, 1/du, 1/dth as double-float (hi, lo)
     // events
     double r_capture;             // r_h (1 + horizon_eps)

@@ -789,39 +789,63 @@ __device__ __forceinline__ long long tile_pixel(const ImageDesc& d, long long q,
 // estimates the ray's distance from the critical curve in impact parameter
 // (dR/db = -2 b r^2 when xi and eta scale together).  Evaluated in FP32 (the
 // band, ~0.15 M, is ~10^6 times its rounding) from the observer's tetrad as in
-// init_ray; the same code classifies a ray in the scan and in the main pass,
-// so every ray is traced exactly once.
+// init_ray.
+//
+// The kernel of the near-critical rays and the kernel of the others each make
+// this test, and every ray is traced exactly once only if both come to the same
+// answer.  It is therefore written in operations whose rounding IEEE 754 fixes
+// and that no compiler contracts or replaces: no build of it, in whichever kernel
+// and at whichever register cap, can round differently (of the plain expressions,
+// builds with and without contraction differed in 7 of 64 images of 2048^2, by two
+// rays or more each).
 // ---------------------------------------------------------------------------
+// cos(acos(c) / 3), c in [-1, 1], through s = cos(acos(c) / 2) = sqrt((1 + c) / 2):
+// as cos(2/3 acos(s)) it is analytic on [0, 1], where this Chebyshev fit of degree
+// 8 is within 7e-8 in FP32.
+__device__ __forceinline__ float cos_third(float c) {
+    const float s = __fsqrt_rn(__fmul_rn(0.5f, __fadd_rn(1.0f, c)));
+    float p = -0.000639314356f;
+    p = fmaf(p, s, 0.00370768644f);
+    p = fmaf(p, s, -0.0103254933f);
+    p = fmaf(p, s, 0.0196757186f);
+    p = fmaf(p, s, -0.0319612958f);
+    p = fmaf(p, s, 0.0532886572f);
+    p = fmaf(p, s, -0.111095682f);
+    p = fmaf(p, s, 0.577349722f);
+    return fmaf(p, s, 0.5f);
+}
+
 __device__ __forceinline__ bool near_critical(const ImageDesc& d, long long q, float band) {
     const long long p = d.pix_begin + q;
     const long long i = p % d.nx, j = p / d.nx;
-    const float al = (float)d.alpha_min + ((float)i + 0.5f) * (float)d.dalpha;
-    const float be = (float)d.beta_min + ((float)j + 0.5f) * (float)d.dbeta;
+    const float al = fmaf(__fadd_rn((float)i, 0.5f), (float)d.dalpha, (float)d.alpha_min);
+    const float be = fmaf(__fadd_rn((float)j, 0.5f), (float)d.dbeta, (float)d.beta_min);
     const float D = (float)d.r_obs;
-    if (!isfinite(al) || !isfinite(be) || !(fmaf(al, al, be * be) < D * D)) return false;
+    if (!isfinite(al) || !isfinite(be) || !(fmaf(al, al, __fmul_rn(be, be)) < __fmul_rn(D, D))) return false;
     // physical momentum at the observer (ZAMO tetrad, as in init_ray)
     const float iN = (float)d.obs_iN, omN = (float)d.obs_omN;
-    const float pu_th = (be / D) * (float)d.obs_ith;
-    const float pu_ph = fmaf(-al / D, (float)d.obs_iph, omN);
+    const float pu_th = __fmul_rn(__fdiv_rn(be, D), (float)d.obs_ith);
+    const float pu_ph = fmaf(-__fdiv_rn(al, D), (float)d.obs_iph, omN);
     const float gtt = (float)d.obs_g[0], gtp = (float)d.obs_g[1], gthth = (float)d.obs_g[3], gpp = (float)d.obs_g[4];
-    const float E = -fmaf(gtt, iN, gtp * pu_ph);
-    const float Lz = fmaf(gtp, iN, gpp * pu_ph);
-    const float pth = gthth * pu_th;
-    float so, co;
-    sincosf((float)d.theta_obs, &so, &co);
-    const float a = (float)d.a, M = (float)d.M, a2 = a * a;
-    const float Q = fmaf(pth, pth, co * co * (Lz * Lz / (so * so) - a2 * E * E));
-    const float xi = Lz / E, eta = Q / (E * E);
-    const float P = 0.5f * (a2 - xi * xi - eta);
-    const float C = 0.5f * M * (eta + (xi - a) * (xi - a));
-    if (!(P < 0.0f) || !(4.0f * P * P * P + 27.0f * C * C < 0.0f)) return false;     // one real root: no minimum
-    const float m = 2.0f * sqrtf(-P * (1.0f / 3.0f));
-    const float cs = fminf(1.0f, fmaxf(-1.0f, 3.0f * C / (P * m)));
-    const float rm = m * cosf(acosf(cs) * (1.0f / 3.0f));
+    const float E = -fmaf(gtt, iN, __fmul_rn(gtp, pu_ph));
+    const float Lz = fmaf(gtp, iN, __fmul_rn(gpp, pu_ph));
+    const float pth = __fmul_rn(gthth, pu_th);
+    const float a = (float)d.a, M = (float)d.M, a2 = __fmul_rn(a, a), E2 = __fmul_rn(E, E);
+    // Q = p_th^2 + cos^2 (L^2 / sin^2 - a^2 E^2) at the observer
+    const float Q = fmaf(pth, pth, fmaf((float)d.cot2_obs, __fmul_rn(Lz, Lz), -__fmul_rn((float)d.cos2_obs, __fmul_rn(a2, E2))));
+    const float xi = __fdiv_rn(Lz, E), eta = __fdiv_rn(Q, E2);
+    const float xa = __fsub_rn(xi, a);
+    const float P = __fmul_rn(0.5f, __fsub_rn(fmaf(-xi, xi, a2), eta));
+    const float C = __fmul_rn(__fmul_rn(0.5f, M), fmaf(xa, xa, eta));
+    const float P3 = __fmul_rn(__fmul_rn(P, P), P), C27 = __fmul_rn(27.0f, C);
+    if (!(P < 0.0f) || !(fmaf(4.0f, P3, __fmul_rn(C27, C)) < 0.0f)) return false;     // one real root: no minimum
+    const float m = __fmul_rn(2.0f, __fsqrt_rn(__fmul_rn(-P, 1.0f / 3.0f)));
+    const float cs = fminf(1.0f, fmaxf(-1.0f, __fdiv_rn(__fmul_rn(3.0f, C), __fmul_rn(P, m))));
+    const float rm = __fmul_rn(m, cos_third(cs));
     if (!(rm > (float)d.r_plus)) return false;
-    const float R = fmaf(fmaf(fmaf(rm, rm, 2.0f * P), rm, 4.0f * C), rm, -a2 * eta);
-    const float b = sqrtf(fmaxf(fmaf(xi, xi, eta), 1e-12f));
-    return fabsf(R) < band * M * (2.0f * rm * rm * b);
+    const float R = fmaf(fmaf(fmaf(rm, rm, __fmul_rn(2.0f, P)), rm, __fmul_rn(4.0f, C)), rm, -__fmul_rn(a2, eta));
+    const float b = __fsqrt_rn(fmaxf(fmaf(xi, xi, eta), 1e-12f));
+    return fabsf(R) < __fmul_rn(__fmul_rn(band, M), __fmul_rn(__fmul_rn(2.0f, __fmul_rn(rm, rm)), b));
 }
 
 // Initial data from the ZAMO tetrad (paper Sec. 2.2), time-reversed, for the
