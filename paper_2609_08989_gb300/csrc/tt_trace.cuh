@@ -1272,6 +1272,35 @@ static __device__ __noinline__ Floats6 floats6(State y, double dr, double dth) {
     return Floats6{StateF{(float)y.r, (float)y.th, (float)y.pr, (float)y.pth}, (float)dr, (float)dth};
 }
 
+// The prescribed split's error norm: in FP64 from the FP32 step h, the FP32 sums es
+// of the error vector (without its factor h) and the FP64 states.
+static __device__ __noinline__ double split_norm_plain(State y, State yn, StateF es, float h, double atol,
+                                                       double rtol) {
+    FpMul m;
+    const double h64 = (double)h;
+    const State e = State{(double)es.r * h64, (double)es.th * h64, (double)es.pr * h64, (double)es.pth * h64};
+    return err_norm2(y, yn, e, atol, rtol, 1.0, m);
+}
+
+// With conversions and products on the integer pipes where they apply: not to sums
+// that are infinite or NaN (a flow at the new point that is, as on the axis), whose
+// norm has to be so too and end the ray.
+__device__ __forceinline__ double split_norm(const State& y, const State& yn, const StateF& es, float h,
+                                             const SolverDesc& sol) {
+    if (sol.int_mul && fabsf(es.r) + fabsf(es.th) + fabsf(es.pr) + fabsf(es.pth) < __int_as_float(0x7f800000)) {
+        IntMul m;
+        const double h64 = int_to_double(h);
+        m.see(yn.r);
+        m.see(yn.pr);
+        m.see(h64);
+        const State e = State{m.chkw(int_to_double(es.r), h64), m.chkw(int_to_double(es.th), h64),
+                              m.chkw(int_to_double(es.pr), h64), m.chkw(int_to_double(es.pth), h64)};
+        const double err = err_norm2(y, yn, e, sol.atol, sol.rtol, 1.0, m);
+        if (m.ok()) return err;
+    }
+    return split_norm_plain(y, yn, es, h, sol.atol, sol.rtol);
+}
+
 template <int PREC, class Lane>
 __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
     constexpr int ACC = (PREC == 2) ? 1 : 0;
@@ -1355,20 +1384,7 @@ __device__ int step_ray32(Lane& L, StateF& yhi, const SolverDesc& sol) {
         // FP64 norm from the FP32 error terms and the FP64 states
         y64n = State{L.y.r + int_to_double(inc.r), L.y.th + int_to_double(inc.th), L.y.pr + int_to_double(inc.pr),
                      L.y.pth + int_to_double(inc.pth)};
-        const double h64 = int_to_double(h);
-        const State es = State{int_to_double(TT_ES(r)), int_to_double(TT_ES(th)), int_to_double(TT_ES(pr)),
-                               int_to_double(TT_ES(pth))};
-        IntMul m;
-        m.see(y64n.r);
-        m.see(y64n.pr);
-        m.see(h64);
-        const State e64 = State{m.chkw(es.r, h64), m.chkw(es.th, h64), m.chkw(es.pr, h64), m.chkw(es.pth, h64)};
-        err64 = err_norm2(L.y, y64n, e64, sol.atol, sol.rtol, 1.0, m);
-        if (!(m.ok() && sol.int_mul)) {
-            FpMul f;
-            const State ef = State{es.r * h64, es.th * h64, es.pr * h64, es.pth * h64};
-            err64 = err_norm2(L.y, y64n, ef, sol.atol, sol.rtol, 1.0, f);
-        }
+        err64 = split_norm(L.y, y64n, StateF{TT_ES(r), TT_ES(th), TT_ES(pr), TT_ES(pth)}, h, sol);
         err2 = nan_bits(err64) ? __int_as_float(0x7fffffff) : (le_pos(err64, 1.0) ? 0.0f : 2.0f);
     } else {
         const float atol = (float)sol.atol, rtol = (float)sol.rtol;
