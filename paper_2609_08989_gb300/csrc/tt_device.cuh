@@ -106,7 +106,8 @@ struct State {
 // formed by m (tt_soft64.cuh).  For IntMul the checks leave every product that
 // is not checked itself with two factors that are normal: r, p_r, s, c and SD
 // lie in 2^+-100, so Sigma, Delta, 1/Sigma, 1/Delta and 1/sin^2 lie in 2^+-300.
-// K cancels to ~1e-16 of its terms, at times to zero.
+// K cancels to ~1e-16 of its terms, at times to zero; p_theta and t2 (without spin
+// p_phi^2 / sin^4) may be zero or tiny.
 template <class Mul>
 __device__ __forceinline__ void kerr_flow64_sc(const KerrK& k, const RayConst& R, const State& y, double s,
                                                double c, State& f, double& H, Mul& m) {
@@ -140,9 +141,9 @@ __device__ __forceinline__ void kerr_flow64_sc(const KerrK& k, const RayConst& R
     const double t1 = fma(-R.pph2, m.mul(u, u), R.a2pt2);
     const double t2 = fma(k.a2, H2, t1);
     f.r = m.mul(m.mul(Del, y.pr), iS);
-    f.th = m.chk(y.pth, iS);
+    f.th = m.chkw(y.pth, iS);
     f.pr = m.chk(fma(r, q1, m.neg(m.chk(r - k.M, q2))), iS);
-    f.pth = m.chk(m.neg(m.mul(sc, iS)), t2);
+    f.pth = m.chkw(t2, m.neg(m.mul(sc, iS)));
 }
 
 __device__ __forceinline__ void kerr_flow64(const KerrK& k, const RayConst& R, const State& y, State& f,
@@ -159,12 +160,16 @@ __device__ __forceinline__ void kerr_flow64(const KerrK& k, const RayConst& R, c
 // against ~28 for a full sincos (measured on GB300); through d^5 and d^6 for
 // |d| < 0.01 (truncation below 2e-18, three fused multiply-adds fewer); farther
 // away, sincos.  (The tier thresholds are compared on the integer pipe.)
-// (theta = theta0, d = 0, fails IntMul's check of sin d.)
+// (theta stays put, d = 0, in the equatorial plane: the series' integer form takes
+// no zero.)
 template <class Mul>
 __device__ __forceinline__ void sincos_near(double th, double th0, double s0, double c0, double& s, double& c,
                                             Mul& m) {
     const double d = th - th0;
-    if (Mul::kInt && abs_below_hi(d, kHi0p01)) {
+    if (Mul::kInt && ((__double2hiint(d) << 1) | __double2loint(d)) == 0) {
+        s = s0;
+        c = c0;
+    } else if (Mul::kInt && abs_below_hi(d, kHi0p01)) {
         // the series below in significands: every term is smaller than its
         // constant and of the other sign, so each sum stays in a binade that is
         // known (the LSB of 1/6 - .. is 2^-55, of 1/24 - .. 2^-57, of 1/2 - .. 2^-54,
@@ -421,7 +426,8 @@ __device__ __forceinline__ void table_fields64(const ImageDesc& d, double r, dou
 // Flow of H = 1/2 [W/D + g^rr p_r^2 + p_th^2 / g_thth], with the inverse of the
 // (t, phi) block, D = g_tt g_phiphi - g_tphi^2,
 // W = g_phiphi p_t^2 - 2 g_tphi p_t p_phi + g_tt p_phi^2.  (For IntMul the fields
-// and p_r are checked; g_tphi, p_phi, p_th and derivatives may be zero.)
+// and p_r are checked; g_tphi, p_phi, p_th and derivatives may be zero; a stage with
+// p_th = 0 exactly where d(g_thth) is not fails.)
 template <class Mul>
 __device__ __forceinline__ void table_flow64(const ImageDesc& d, const RayConst& R, const State& y,
                                              State& f, double& H, Mul& m) {
@@ -433,26 +439,26 @@ __device__ __forceinline__ void table_flow64(const ImageDesc& d, const RayConst&
     m.see(F[4]);
     m.see(y.pr);
     m.see(R.pt);
-    const double pt2 = m.mul(R.pt, R.pt), ptp = m.mulz(R.pph, R.pt2);
+    const double pt2 = m.mul(R.pt, R.pt), ptp = m.chkw(R.pph, R.pt2);
     double D = fma(F[0], F[3], m.neg(m.mulz(F[1], F[1])));
     double iD = rcp64(D);
-    double W = fma(F[3], pt2, fma(-F[1], ptp, m.mulz(R.pph2, F[0])));
+    double W = fma(F[3], pt2, fma(-F[1], ptp, m.chkw(R.pph2, F[0])));
     double WiD = m.mulz(W, iD);
     double ith = rcp64(F[2]);
     double pr2 = m.mul(y.pr, y.pr), pth2 = m.chkw(y.pth, y.pth);
     H = 0.5 * (WiD + fma(F[4], pr2, m.chkw(pth2, ith)));
-    double dW_r = fma(Fr[3], pt2, fma(-Fr[1], ptp, m.mulz(R.pph2, Fr[0])));
+    double dW_r = fma(Fr[3], pt2, fma(-Fr[1], ptp, m.chkw(R.pph2, Fr[0])));
     const double m2F1 = m.mulz(F[1], -2.0);
     double dD_r = fma(Fr[0], F[3], fma(F[0], Fr[3], m.mulz(m2F1, Fr[1])));
-    double dW_t = fma(Ft[3], pt2, fma(-Ft[1], ptp, m.mulz(R.pph2, Ft[0])));
+    double dW_t = fma(Ft[3], pt2, fma(-Ft[1], ptp, m.chkw(R.pph2, Ft[0])));
     double dD_t = fma(Ft[0], F[3], fma(F[0], Ft[3], m.mulz(m2F1, Ft[1])));
     double ith2 = m.mul(ith, ith);
-    double d2H_r = fma(fma(-WiD, dD_r, dW_r), iD, fma(Fr[4], pr2, m.chkw(m.mulz(m.neg(Fr[2]), ith2), pth2)));
-    double d2H_t = fma(fma(-WiD, dD_t, dW_t), iD, fma(Ft[4], pr2, m.chkw(m.mulz(m.neg(Ft[2]), ith2), pth2)));
+    double d2H_r = fma(fma(-WiD, dD_r, dW_r), iD, fma(Fr[4], pr2, m.chkw(m.chkw(m.neg(Fr[2]), ith2), pth2)));
+    double d2H_t = fma(fma(-WiD, dD_t, dW_t), iD, fma(Ft[4], pr2, m.chkw(m.chkw(m.neg(Ft[2]), ith2), pth2)));
     f.r = m.mul(F[4], y.pr);
-    f.th = m.mulz(y.pth, ith);
+    f.th = m.chkw(y.pth, ith);
     f.pr = m.mulz(d2H_r, -0.5);
-    f.pth = m.mulz(d2H_t, -0.5);
+    f.pth = m.chkw(d2H_t, -0.5);
 }
 
 __device__ __forceinline__ void table_lower64(const ImageDesc& d, double r, double th, double g[5]) {

@@ -157,11 +157,21 @@ __device__ __forceinline__ float int_to_float(double x) {
 //   neg(x)     -x
 //   mulz(a, b) the product where a may be zero
 //   chkw(a, b) the same, whose magnitude is to be zero or in 2^-400 .. 2^400
+//   seew(x)    x, which is to be zero or in 2^-400 .. 2^400
+//   rest(a, b) the product of an a that seew has taken and a constant
+// p_phi, p_theta and what follows from them are zero or tiny in earnest (the column
+// alpha = 0 of an image, the equatorial plane, a metric without spin), for whole
+// rays: they take the wide forms, since one lane that fails its checks at every
+// attempt makes its warp run both kinds of attempt (a 97 x 61 table image of odd
+// width, with such a column, 220 ms; 127 with the wide forms, 138 with plain attempts
+// alone; 65536 equatorial rays 18.0, 9.3 and 17.3 ms).
 struct FpMul {
     static constexpr bool kInt = false;
     __device__ __forceinline__ double neg(double x) { return -x; }
     __device__ __forceinline__ double mulz(double a, double b) { return a * b; }
     __device__ __forceinline__ double chkw(double a, double b) { return a * b; }
+    __device__ __forceinline__ double rest(double a, double b) { return a * b; }
+    __device__ __forceinline__ void seew(double) {}
     __device__ __forceinline__ double mul(double a, double b) { return a * b; }
     __device__ __forceinline__ double chk(double a, double b) { return a * b; }
     __device__ __forceinline__ void see(double) {}
@@ -176,18 +186,30 @@ struct IntMul {
         return __hiloint2double(__double2hiint(x) ^ 0x80000000, __double2loint(x));
     }
     unsigned bad = 0;
+    static __device__ __forceinline__ bool is_zero(double x) {
+        return ((__double2hiint(x) << 1) | __double2loint(x)) == 0;
+    }
+    static __device__ __forceinline__ double zero_of(double a, double b) {
+        return __hiloint2double((__double2hiint(a) ^ __double2hiint(b)) & 0x80000000, 0);
+    }
+    // the exponent field relative to 2^-400, in the units of see()'s bound
+    __device__ __forceinline__ void wide(unsigned hi) { bad = max(bad, (hi + hi - ((1023u - 400u) << 21)) >> 2); }
     __device__ __forceinline__ double mulz(double a, double b) {
-        const bool zero = ((__double2hiint(a) << 1) | __double2loint(a)) == 0;
+        const bool zero = is_zero(a);
         const double p = soft_mul64(a, b);
         see(zero ? 1.0 : p);
-        return zero ? __hiloint2double((__double2hiint(a) ^ __double2hiint(b)) & 0x80000000, 0) : p;
+        return zero ? zero_of(a, b) : p;
     }
     __device__ __forceinline__ double chkw(double a, double b) {
-        const bool zero = ((__double2hiint(a) << 1) | __double2loint(a)) == 0;
+        const bool zero = is_zero(a);
         const double p = soft_mul64(a, b);
-        const unsigned hi = zero ? 1023u << 20 : (unsigned)__double2hiint(p);
-        bad = max(bad, (hi + hi - ((1023u - 400u) << 21)) >> 2);
-        return zero ? __hiloint2double((__double2hiint(a) ^ __double2hiint(b)) & 0x80000000, 0) : p;
+        wide(zero ? 1023u << 20 : (unsigned)__double2hiint(p));
+        return zero ? zero_of(a, b) : p;
+    }
+    __device__ __forceinline__ void seew(double x) { wide(is_zero(x) ? 1023u << 20 : (unsigned)__double2hiint(x)); }
+    __device__ __forceinline__ double rest(double a, double b) {
+        const double p = soft_mul64(a, b);
+        return is_zero(a) ? zero_of(a, b) : p;
     }
     __device__ __forceinline__ double mul(double a, double b) { return soft_mul64(a, b); }
     __device__ __forceinline__ double chk(double a, double b) {

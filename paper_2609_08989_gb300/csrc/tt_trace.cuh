@@ -120,7 +120,7 @@ __device__ __forceinline__ State plus(const State& y, double h, const State& k) 
 
 template <class Mul>
 __device__ __forceinline__ State times(const State& k, double w, Mul& m) {
-    return State{m.mul(k.r, w), m.mul(k.th, w), m.mul(k.pr, w), m.mul(k.pth, w)};
+    return State{m.mul(k.r, w), m.rest(k.th, w), m.mul(k.pr, w), m.rest(k.pth, w)};
 }
 
 template <int METRIC, int METHOD, class Mul>
@@ -133,9 +133,9 @@ __device__ __forceinline__ void rk_step64(const ImageDesc& d, const KerrK& kk, c
     cn = c0;
     m.see(h);
     m.see(k1.r);
-    m.see(k1.th);
+    m.seew(k1.th);
     m.see(k1.pr);
-    m.see(k1.pth);
+    m.seew(k1.pth);
     if (METRIC == 0) {
         m.see(s0);
         m.see(c0);
