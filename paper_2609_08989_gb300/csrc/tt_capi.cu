@@ -259,9 +259,9 @@ tt::SolverDesc make_solver(const tt_solver* s) {
     sd.refine = s->refine;
     sd.precision = s->precision;
     sd.method = s->method;
-    // products of the error norm's scale factors stay far inside the normal range
-    auto mid = [](double x) { return x >= 0x1p-47 && x <= 0x1p47; };
-    sd.int_mul = mid(s->rtol) && mid(s->atol);
+    // the error norm's scale factors stay far inside the normal range (an absolute
+    // tolerance next to zero, for a relative one alone, does not matter)
+    sd.int_mul = s->rtol <= 0x1p47 && s->atol <= 0x1p47 && (s->rtol >= 0x1p-90 || s->atol >= 0x1p-90);
     // near-critical rays in double-float: mixed paths only (default band 0.15 M,
     // none on the prescribed split), at the FP64 path's tolerance by default
     sd.crit_band = 0.0;

@@ -85,7 +85,8 @@ struct SolverDesc {
     int refine;                   // 0 Henon, 1 Hermite, 2 Henon in FP64 on the mixed paths too
     int precision;                // 0 FP64, 1 mixed (FP64 state), 2 mixed (FP32-pair state),
                                   // 3 double-float, 4 mixed with the FP64 norm, zone steps and refinement
-    int int_mul;                  // FP64 pairs: products on the integer pipes (tolerances in range)
+    int int_mul;                  // FP64 steps of one metric kind, and the prescribed split's norm and zone
+                                  // steps: products on the integer pipes (tolerances in range)
     int method;                   // 0 Dormand-Prince; FP64 only: 1 Cash-Karp, 2 Fehlberg, 3 GBS, 4 Verlet
     // mixed paths: rays within crit_band (units of M) of the critical curve are
     // traced in double-float at crit_rtol / crit_atol (0: none)

@@ -157,6 +157,7 @@ __device__ __forceinline__ float int_to_float(double x) {
 //   neg(x)     -x
 //   mulz(a, b) the product where a may be zero
 //   chkw(a, b) the same, whose magnitude is to be zero or in 2^-400 .. 2^400
+//   chkm(a, b) the product, whose magnitude is to lie in 2^-200 .. 2^200
 //   seew(x)    x, which is to be zero or in 2^-400 .. 2^400
 //   rest(a, b) the product of an a that seew has taken and a constant
 // p_phi, p_theta and what follows from them are zero or tiny in earnest (the column
@@ -170,6 +171,7 @@ struct FpMul {
     __device__ __forceinline__ double neg(double x) { return -x; }
     __device__ __forceinline__ double mulz(double a, double b) { return a * b; }
     __device__ __forceinline__ double chkw(double a, double b) { return a * b; }
+    __device__ __forceinline__ double chkm(double a, double b) { return a * b; }
     __device__ __forceinline__ double rest(double a, double b) { return a * b; }
     __device__ __forceinline__ void seew(double) {}
     __device__ __forceinline__ double mul(double a, double b) { return a * b; }
@@ -205,6 +207,12 @@ struct IntMul {
         const double p = soft_mul64(a, b);
         wide(zero ? 1023u << 20 : (unsigned)__double2hiint(p));
         return zero ? zero_of(a, b) : p;
+    }
+    __device__ __forceinline__ double chkm(double a, double b) {
+        const double p = soft_mul64(a, b);
+        const unsigned hi = (unsigned)__double2hiint(p);
+        bad = max(bad, (hi + hi - ((1023u - 200u) << 21)) >> 1);
+        return p;
     }
     __device__ __forceinline__ void seew(double x) { wide(is_zero(x) ? 1023u << 20 : (unsigned)__double2hiint(x)); }
     __device__ __forceinline__ double rest(double a, double b) {

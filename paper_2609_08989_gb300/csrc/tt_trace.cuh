@@ -345,13 +345,6 @@ __device__ __forceinline__ double sq3(double a, double b, double c) {
     return fma(c, c, fma(b, b, a * a));
 }
 
-// Mean-square error norm over (r, theta, p_r, p_theta).  The four scale
-// factors share one reciprocal: 1/sc_0 = sc_1 sc_2 sc_3 / (sc_0 sc_1 sc_2 sc_3),
-// refined by a single Newton step (~1e-14 relative: the norm only decides
-// err <= 1 and scales the step).  A product outside the normal range (tolerances
-// near 1e-75 or 1e75) takes the per-component reciprocals instead.
-// The error vector is he * e (he = h for the Runge-Kutta pairs, whose e omits
-// the step's factor h; 1 otherwise).
 // max(|a|, |b|) of two doubles that are not NaN, on the integer pipe (fmax takes
 // two FP64 issue slots: magnitudes order as their bit patterns).
 __device__ __forceinline__ double max_abs(double a, double b) {
@@ -360,10 +353,19 @@ __device__ __forceinline__ double max_abs(double a, double b) {
     return __longlong_as_double((long long)max(x, y));
 }
 
-// (yn may hold a NaN or an infinity only where the caller then ends the ray,
-// whatever the norm.)  For IntMul: the tolerances lie in 2^+-47 (the caller's
-// condition), so every scale factor is at least 2^-47, and those of r and p_r
-// are bounded by the flow's checks of yn; he is checked by rk_step64.
+// Mean-square error norm over (r, theta, p_r, p_theta).  The four scale
+// factors share one reciprocal: 1/sc_0 = sc_1 sc_2 sc_3 / (sc_0 sc_1 sc_2 sc_3),
+// refined by a single Newton step (~1e-14 relative: the norm only decides
+// err <= 1 and scales the step).  A product outside the normal range (tolerances
+// near 1e-75 or 1e75) takes the per-component reciprocals instead.
+// The error vector is he * e (he = h for the Runge-Kutta pairs, whose e omits
+// the step's factor h; 1 otherwise).
+//
+// yn may hold a NaN or an infinity only where the caller then ends the ray,
+// whatever the norm.  For IntMul: one of the tolerances is at least 2^-90 and both
+// at most 2^47 (SolverDesc::int_mul), and |r| and |p_r| of yn lie in 2^+-100 (the
+// flow's checks), so that the scale factors of r and p_r lie in 2^+-190; the checks
+// of p01 and p23 bound the other two.  he is checked by the caller.
 template <class Mul>
 __device__ __forceinline__ double err_norm2(const State& y, const State& yn, const State& e,
                                             double atol, double rtol, double he, Mul& m) {
@@ -371,7 +373,7 @@ __device__ __forceinline__ double err_norm2(const State& y, const State& yn, con
     const double s1 = fma(rtol, max_abs(y.th, yn.th), atol);
     const double s2 = fma(rtol, max_abs(y.pr, yn.pr), atol);
     const double s3 = fma(rtol, max_abs(y.pth, yn.pth), atol);
-    const double p01 = m.chk(s0, s1), p23 = m.chk(s2, s3);
+    const double p01 = m.chkm(s0, s1), p23 = m.chkm(s2, s3);
     const double pp = m.mul(p01, p23);
     // outside [2^-930, 2^930] (the exponent field, on the integer pipe)
     const int ex = (__double2hiint(pp) >> 20) & 0x7ff;
