@@ -439,7 +439,7 @@ def other_paths(T, args, flush, peaks, main_sc):
     objs["batch"] = {"value": rays / (ms / 1e3), "unit": UNIT, "ms_per_replay": ms, "rays": rays,
                      "workload": "batch_uneven_64_images_seed2609_mixed_pair", "images": 64,
                      "res": [min(s.nx for s in imgs), max(s.nx for s in imgs)], "rtol": imgs[0].rtol,
-                     "launch": "CUDA graph replay of one tartarus_trace_batch call (%d launch)"
+                     "launch": "CUDA graph replay of one tartarus_trace_batch call (%d kernels)"
                                % graph.launches_per_replay,
                      "rk_step_attempts": batt, "h_max_escaped": hesc,
                      "roofline": fp32_roofline(batt, ms, peaks)}

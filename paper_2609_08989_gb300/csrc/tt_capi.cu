@@ -280,6 +280,9 @@ tt::SolverDesc make_solver(const tt_solver* s) {
     return sd;
 }
 
+// Kernels per launch: the mixed paths' near-critical rays have one of their own.
+int kernels_of(const tt::SolverDesc& sd) { return sd.crit_band > 0.0 ? 2 : 1; }
+
 tt::LaunchShape make_shape(const tt_tune* t) {
     tt::LaunchShape s{0, 0, 0, 0, 0, 0, 0, 0, 0, 0};       // zeros: the kernel's defaults
     if (t) {
@@ -391,7 +394,7 @@ int enqueue(const std::vector<tt::ImageDesc>& descs, const tt_solver* sol, const
         cudaError_t e = cudaMemsetAsync(q, 0, 2 * sizeof(unsigned long long), st);
         if (e == cudaSuccess) e = tt::launch_trace(ds, (int)n, total, metric_mode, sd, shape, q, st);
         if (e != cudaSuccess) return TT_ECUDA;
-        g_launches.fetch_add(1);
+        g_launches.fetch_add(kernels_of(sd));
     }
     return TT_OK;
 }
@@ -484,7 +487,7 @@ int tartarus_trace_batch_noalloc(const tt_image* images, int n, const tt_solver*
             cudaError_t e = cudaMemsetAsync(q, 0, 2 * sizeof(unsigned long long), st);
             if (e == cudaSuccess) e = tt::launch_trace(ds, nd, total, metric_mode, sd, shape, q, st);
             if (e != cudaSuccess) return TT_ECUDA;
-            g_launches.fetch_add(1);
+            g_launches.fetch_add(kernels_of(sd));
             nd = 0;
             total = 0;
             n_table = 0;

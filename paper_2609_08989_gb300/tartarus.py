@@ -433,9 +433,10 @@ class TraceGraph:
         torch.cuda.current_stream().wait_stream(side)
         torch.cuda.synchronize()
         self.graph = torch.cuda.CUDAGraph()
+        before = launch_count()
         with torch.cuda.graph(self.graph):
             trace_batch(self.scenes, self.outs, stream=torch.cuda.current_stream(), tune=tune, tables=tables)
-        self.launches_per_replay = (len(self.scenes) + 63) // 64
+        self.launches_per_replay = launch_count() - before        # kernels
 
     def replay(self):
         self.graph.replay()

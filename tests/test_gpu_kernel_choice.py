@@ -34,3 +34,29 @@ def test_build_by_number_of_rays(images, side, few):
     assert len(names) == (images + 63) // 64, names
     for n in names:
         assert ("trace_kernel64<" in n) == few and ("regcap" in n) == (not few), names
+
+
+@pytest.mark.parametrize("precision,band,each", [(scenes.FP64, 0.0, 1), (scenes.DOUBLE_FLOAT, 0.0, 1),
+                                                 (scenes.MIXED, 0.0, 2), (scenes.MIXED_PAIR, 0.0, 2),
+                                                 (scenes.MIXED_PAIR, -1.0, 1), (scenes.MIXED_SPLIT, 0.0, 1),
+                                                 (scenes.MIXED_SPLIT, 0.15, 2)])
+def test_launch_count_counts_kernels(precision, band, each):
+    """The near-critical rays of the mixed paths run in a kernel of their own, which
+    tartarus_launch_count and a graph's launches_per_replay count too."""
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    from paper_2609_08989_gb300 import tartarus as T
+    sc = scenes.kerr_disk(24, precision).replace(rtol=1e-7, atol=1e-7, critical_band=band)
+    out = T.alloc_outputs(sc.npix)
+    n0 = T.launch_count()
+    T.trace(sc, out=out)
+    assert T.launch_count() - n0 == each
+    assert len(kernels(lambda: T.trace(sc, out=out))) == each
+    imgs = [sc] * 65
+    outs = [T.alloc_outputs(sc.npix) for _ in imgs]
+    n0 = T.launch_count()
+    status = []
+    T.trace_batch_noalloc(imgs, outs, status_out=status)
+    assert T.launch_count() - n0 == 2 * each and status == [0] * 65
+    assert T.TraceGraph(imgs, outs).launches_per_replay == 2 * each
+    torch.cuda.synchronize()
