@@ -186,13 +186,23 @@ def config_dict(sc, world, shard=False):
             "l2": "flushed between timed steps (256 MiB write); working set is a few MB of state + outputs"}
 
 
-def kernel_name(sc):
-    """The tracing kernel the FP64 launch of this scene runs (its tuned block size)."""
+def kernel_name(sc, rays=None):
+    """The tracing kernel that an FP64 launch of this scene runs: by its tuned shape, and
+    by whether every ray has a lane of its own (launch64, launch_rk_n)."""
+    import torch
     from paper_2609_08989_gb300 import autotune
-    block = (autotune.cached(sc) or {}).get("block", 0)
+    tune = autotune.cached(sc) or {}
+    block, regs = tune.get("block", 0), tune.get("reg_variant", 0)
+    few = (sc.npix if rays is None else rays) <= 2 * 128 * torch.cuda.get_device_properties(0).multi_processor_count
     if sc.method == 0:
-        return {256: "trace_kernel64_b256<0,1>", 384: "trace_kernel64_b384<0,1>"}.get(block, "trace_kernel64<0,1>")
-    return "trace_kernel_rk<%d,0,1,%d>" % (sc.method, 256 if block in (256, 384) else 128)
+        if block in (256, 384):
+            return "trace_kernel64_b%d<0,1>" % block
+        if few and regs == 0:
+            return "trace_kernel64<0,1>"
+        return "trace_kernel64_regcap<%d,1>" % (4 if regs == 2 else 3)
+    if block in (256, 384):
+        return "trace_kernel_rk<%d,0,1,256,1>" % sc.method
+    return "trace_kernel_rk<%d,0,1,128,%d>" % (sc.method, 1 if few or sc.method > 2 else 3)
 
 
 def h_stats(out):
@@ -643,7 +653,7 @@ def run_tartarus(args):
                          "traffic": (TRAFFIC_BYTES_1024 * count / (1024 * 1024)
                                      if TRAFFIC_BYTES_1024 and args.precision == "fp64" and sc.method == 0 else None),
                          "traffic_note": "DRAM bytes of one full-size launch (ncu), scaled by the pixels traced",
-                         "kernel": kernel_name(sc), "kernel_ms": mean_kern,
+                         "kernel": kernel_name(sc, count), "kernel_ms": mean_kern,
                          "flops_per_unit": fpu,
                          "unit_of_work": "%s step attempt" % METHOD_NAMES[sc.method],
                          "issued": ({"fp64_flops_per_unit": issued,

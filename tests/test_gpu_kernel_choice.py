@@ -60,3 +60,16 @@ def test_launch_count_counts_kernels(precision, band, each):
     assert T.launch_count() - n0 == 2 * each and status == [0] * 65
     assert T.TraceGraph(imgs, outs).launches_per_replay == 2 * each
     torch.cuda.synchronize()
+
+
+@pytest.mark.parametrize("method", [scenes.DOPRI5, scenes.CASH_KARP, scenes.GBS])
+@pytest.mark.parametrize("side", [16, 256])
+def test_benchmark_names_the_kernel(method, side):
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import bench
+    from paper_2609_08989_gb300 import tartarus as T
+    sc = scenes.kerr_disk(side).replace(method=method, rtol=1e-6, atol=1e-6)
+    out = T.alloc_outputs(sc.npix)
+    names = kernels(lambda: T.trace(sc, out=out))
+    assert len(names) == 1 and bench.kernel_name(sc) in names[0].replace(" ", ""), (names, bench.kernel_name(sc))
