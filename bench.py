@@ -86,9 +86,9 @@ TABLE_DF_FP32_INST_PER_STEP = 15398
 MIXED_FP32_INST_PER_STEP = 889
 BYTES_OUT_PER_PIXEL = 3 * 3 * 8 + 8 + 8 + 4 + 4 + 1 + 1
 # DRAM traffic of the FP64 tracer per launch on the 1024^2 image: ncu's
-# dram__bytes_read.sum + dram__bytes_write.sum of one full-size launch (2.6 MB read,
-# 51.2 MB written: part of the 103 MB of outputs leaves the L2 during the kernel)
-TRAFFIC_BYTES_1024 = 2555392 + 51188480
+# dram__bytes_read.sum + dram__bytes_write.sum of one full-size launch (3.81 MB read,
+# 51.70 MB written: part of the 103 MB of outputs leaves the L2 during the kernel)
+TRAFFIC_BYTES_1024 = 3810000 + 51700000
 # host-to-device input of one step: the launch's parameter block (sizeof(tt::LaunchParams<1>):
 # solver settings, launch shape and the image descriptor)
 DESC_BYTES = 736

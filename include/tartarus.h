@@ -219,10 +219,10 @@ typedef struct {
  *                   mixed paths 256 (default; 384 runs as 256, 128 fails with
  *                   TT_ECUDA).  Other sizes: TT_EUNSUPPORTED.
  *   reg_variant     registers per thread of the FP64 closed-form Kerr kernel at
- *                   128 threads, single camera: 0 by the number of rays (the
- *                   compiler's choice where every ray has a lane of its own, at
- *                   most 168 otherwise), 1 at most 168, 2 at most 128 (other
- *                   kernels ignore it)
+ *                   128 threads: 0 by the number of rays (the compiler's choice
+ *                   where every ray has a lane of its own, at most 168
+ *                   otherwise), 1 at most 168, 2 at most 128 (1 and 2 for a
+ *                   single camera; batches and other kernels ignore them)
  *   refill          flush finished rays and refill lanes once at least this many
  *                   lanes of a warp are done or idle (1..32; default 32)
  *   blocks_per_sm   persistent blocks per SM (0: as many as fit)

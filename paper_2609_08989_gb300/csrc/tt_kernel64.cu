@@ -13,7 +13,7 @@ __global__ void __launch_bounds__(256) trace_kernel64_b256(const __grid_constant
     trace_loop<METRIC, 0>(p.desc, p.n_desc, p.total, p.sol, p.tune, p.queue);
 }
 
-// 384 threads (12 warps per SM at 160 registers, against 8 for 256 threads).
+// 384 threads (12 warps per SM at 168 registers, against 8 for 256 threads).
 template <int METRIC, int N>
 __global__ void __launch_bounds__(384) trace_kernel64_b384(const __grid_constant__ LaunchParams<N> p) {
     trace_loop<METRIC, 0>(p.desc, p.n_desc, p.total, p.sol, p.tune, p.queue);
@@ -50,11 +50,11 @@ static cudaError_t launch64(const ImageDesc* descs, int n, long long total, int 
     if (metric_mode == 0) {
         if (shape.block == 256) return launch_persistent<N>(trace_kernel64_b256<0, N>, 256, bps, p, stream);
         if (shape.block == 384) return launch_persistent<N>(trace_kernel64_b384<0, N>, 384, bps, p, stream);
-        // the uncapped build (two blocks per SM, no spills) where every ray has a lane of
-        // its own, so that the longest ray sets the time (64^2 shadow 10.0 ms, capped
-        // 11.2; a batch of 64 images of 16^2 8.2 ms, capped 9.0); else three blocks per
-        // SM (1024^2 disk 152.1 ms, uncapped 157.7): the FP64 unit then waits less for
-        // warps that are in their integer products
+        // the uncapped build (202 registers, two blocks per SM, no spills) where every
+        // ray has a lane of its own, so that the longest ray sets the time (64^2 shadow
+        // 10.1 ms, capped 11.0; a batch of 64 images of 16^2 8.2 ms, capped 9.0); else
+        // three blocks per SM (1024^2 disk 153.9 ms, uncapped 157.0): the FP64 unit then
+        // waits less for warps that are in their integer products
         if ((N > 1 || shape.reg_variant == 0) && total <= 2LL * 128 * sm_count())
             return launch_persistent<N>(trace_kernel64<0, N>, 128, bps, p, stream);
         if constexpr (N == 1) {

@@ -5,7 +5,7 @@
 
 namespace tt {
 
-// One 256-thread block per SM at ~186 registers, no spills.  The kernel of the
+// One 256-thread block per SM at 198 (FP32 pair) or 204 registers, no spills.  The kernel of the
 // other rays may start once these blocks are resident (programmatic dependent
 // launch): it takes the SMs as they end, so that the tail of the longest rays
 // (up to ~1200 step attempts of ~6 us) runs beside it.  Fewer SMs for these rays

@@ -6,7 +6,7 @@
 
 namespace tt {
 
-// 256-thread blocks, registers uncapped (~180: one block per SM; a cap at 128
+// 256-thread blocks, registers uncapped (201: one block per SM; a cap at 128
 // spills and measured 10 % slower).
 template <int METRIC, int N>
 __global__ void __launch_bounds__(256) trace_kernel_df(const __grid_constant__ LaunchParams<N> p) {

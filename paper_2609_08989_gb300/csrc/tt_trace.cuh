@@ -753,9 +753,13 @@ __device__ __forceinline__ long long outward(long long k, long long n, long long
 // rays per lane the last of them run on a GPU that is otherwise empty: the
 // double-float table image of 512^2 (6.7 rays per lane) 310 -> 268 ms, of 768^2
 // 560 -> 491 ms; FP64 384^2 32.3 -> 29.0 ms, double-float 256^2 6.4 -> 5.3 ms, the
-// prescribed split's 1024^2 35.1 -> 32.2 ms; no change with many.  Where every ray
-// has a lane from the start there is no order to gain from, and narrow images
-// lost (33 x 299 table 59 -> 63 ms): launches of at most 256 rays per SM keep the
+// prescribed split's 1024^2 35.1 -> 32.2 ms; no change with many.  The first gains
+// show at 431 rays per SM (256^2 FP64 table image 103 -> 90 ms, double-float 6.2 ->
+// 5.15 ms; none at 330).  Where every ray has a lane from the start there is no order
+// to gain from: of 19 images of at most 256 rays per SM, twenty runs each way, 18
+// differed by less than the runs of one side (up to 30 % on narrow table images, where
+// chance decides which long rays share a scheduler) and one was slower from the middle
+// (147 x 201 double-float table, medians 46.4 and 50.3 ms).  Such launches keep the
 // order of beta.  The mixed kernels whose near-critical rays run apart have no such
 // tail, and are 2-10 % slower when the rays that need zone steps come all at
 // once (768^2 8.8 -> 9.8 ms, 2048^2 38.1 -> 39.1 ms): they keep the order of beta.
@@ -1156,10 +1160,10 @@ __device__ int step_ray64(Lane& L, const SolverDesc& sol) {
     if constexpr (METRIC != 2 && (PREC == 0 || PREC == 4)) {
         // products on the integer pipes (the FP64 unit, 87 % busy, was the bound:
         // with these and the integer series of sin and cos the 1024^2 disk takes
-        // 152.9 instead of 258.8 ms); where their operands leave the checked range (a
+        // 153.9 instead of 258.8 ms); where their operands leave the checked range (a
         // stage inside the horizon) the attempt is made again with plain products,
-        // and a ray whose operands leave it at every attempt (one that stays in the
-        // equatorial plane, p_theta = 0) goes on with plain products alone
+        // and a ray whose operands leave it at every attempt (one that starts at r >
+        // 2^25) goes on with plain products alone
         if ((sol.int_mul || METHOD == 4) && L.plain_run < kPlainRun) {
             IntMul m;
             if constexpr (METHOD == 4) {
