@@ -450,7 +450,7 @@ __device__ __forceinline__ void table_flow64(const ImageDesc& d, const RayConst&
     double dW_r = fma(Fr[3], pt2, fma(-Fr[1], ptp, m.chkw(R.pph2, Fr[0])));
     const double m2F1 = m.mulz(F[1], -2.0);
     double dD_r = fma(Fr[0], F[3], fma(F[0], Fr[3], m.mulz(m2F1, Fr[1])));
-    double dW_t = fma(Ft[3], pt2, fma(-Ft[1], ptp, m.chkw(R.pph2, Ft[0])));
+    double dW_t = fma(Ft[3], pt2, fma(-Ft[1], ptp, m.chkz(R.pph2, Ft[0])));
     double dD_t = fma(Ft[0], F[3], fma(F[0], Ft[3], m.mulz(m2F1, Ft[1])));
     double ith2 = m.mul(ith, ith);
     double d2H_r = fma(fma(-WiD, dD_r, dW_r), iD, fma(Fr[4], pr2, m.chkw(m.chkw(m.neg(Fr[2]), ith2), pth2)));

@@ -157,20 +157,23 @@ __device__ __forceinline__ float int_to_float(double x) {
 //   neg(x)     -x
 //   mulz(a, b) the product where a may be zero
 //   chkw(a, b) the same, whose magnitude is to be zero or in 2^-400 .. 2^400
+//   chkz(a, b) the same where b may be zero too
 //   chkm(a, b) the product, whose magnitude is to lie in 2^-200 .. 2^200
 //   seew(x)    x, which is to be zero or in 2^-400 .. 2^400
 //   rest(a, b) the product of an a that seew has taken and a constant
 // p_phi, p_theta and what follows from them are zero or tiny in earnest (the column
 // alpha = 0 of an image, the equatorial plane, a metric without spin), for whole
 // rays: they take the wide forms, since one lane that fails its checks at every
-// attempt makes its warp run both kinds of attempt (a 97 x 61 table image of odd
-// width, with such a column, 220 ms; 127 with the wide forms, 138 with plain attempts
-// alone; 65536 equatorial rays 18.0, 9.3 and 17.3 ms).
+// attempt, or one ray in 20 at each, makes whole warps run both kinds of attempt (a
+// 97 x 61 table image of odd width, with such a column, 220 ms; 127 with the wide
+// forms, 138 with plain attempts alone; without spin 56, 33.5 and 36.7; 65536
+// equatorial rays 18.0, 9.3 and 17.3 ms).
 struct FpMul {
     static constexpr bool kInt = false;
     __device__ __forceinline__ double neg(double x) { return -x; }
     __device__ __forceinline__ double mulz(double a, double b) { return a * b; }
     __device__ __forceinline__ double chkw(double a, double b) { return a * b; }
+    __device__ __forceinline__ double chkz(double a, double b) { return a * b; }
     __device__ __forceinline__ double chkm(double a, double b) { return a * b; }
     __device__ __forceinline__ double rest(double a, double b) { return a * b; }
     __device__ __forceinline__ void seew(double) {}
@@ -204,6 +207,12 @@ struct IntMul {
     }
     __device__ __forceinline__ double chkw(double a, double b) {
         const bool zero = is_zero(a);
+        const double p = soft_mul64(a, b);
+        wide(zero ? 1023u << 20 : (unsigned)__double2hiint(p));
+        return zero ? zero_of(a, b) : p;
+    }
+    __device__ __forceinline__ double chkz(double a, double b) {
+        const bool zero = is_zero(a) || is_zero(b);
         const double p = soft_mul64(a, b);
         wide(zero ? 1023u << 20 : (unsigned)__double2hiint(p));
         return zero ? zero_of(a, b) : p;
