@@ -11,13 +11,19 @@ torch = pytest.importorskip("torch")
 
 
 def kernels(call):
-    """Names of the tracing kernels that a call launches."""
+    """Names of the tracing kernels that a call launches (skips where the profiler does
+    not list even a kernel of torch's own)."""
     from torch.profiler import ProfilerActivity, profile
+    marker = torch.zeros(1, device="cuda")
     for _ in range(2):          # (the first profile of a process may miss what it starts up with)
         with profile(activities=[ProfilerActivity.CUDA]) as prof:
+            marker.add_(1.0)
             call()
             torch.cuda.synchronize()
-    return [e.name for e in prof.events() if "trace_kernel" in e.name]
+    names = [e.name for e in prof.events()]
+    if not any("elementwise" in n for n in names):
+        pytest.skip("the profiler lists no kernels here")
+    return [n for n in names if "trace_kernel" in n]
 
 
 @pytest.mark.parametrize("images,side,few", [(1, 16, True), (3, 16, True), (65, 8, True), (1, 256, False), (4, 128, False)])
